@@ -93,12 +93,11 @@ struct tpc_tf {
   Args last_args;
   // learned link classifier (TPC_MODE_PRUNED)
   int4 *amb = nullptr;        // clusters listed for rescoring (arena, pruned mode only)
-  PruneRow *q_rows = nullptr; // per-tile regions of rescored pairs (pruned mode only)
+  PruneRec *q_rec = nullptr;  // per-tile regions of ambiguous clusters (pruned mode only)
   int32_t *q_count = nullptr;
   float *rr_feat = nullptr, *rr_logit = nullptr;  // the regions' rows as dense feature rows, their logits
   int4 *rr_meta = nullptr;                        // each dense row's (cluster, j, k)
   int64_t *rr_cost = nullptr;                     // and its cost
-  uint32_t *rr_tbase = nullptr;                   // each region's first dense row
   MlpW *mlp = nullptr;        // packed weights (allocated by tpc_mlp_load)
   MlpHead mlp_head = {};      // host copy of the values every scored row reads
   float *mlp_stage = nullptr; // FP32 blob body staged for packing
@@ -267,15 +266,14 @@ static std::vector<Part> plan_arena(tpc_tf *tf, const tpc_tf_config *cfg) {
       {(void **)&tf->r_status, (size_t)tf->track_list_cap},
       {(void **)&tf->h_ntracks, 16},
       {(void **)&tf->amb, cfg->mode == TPC_MODE_PRUNED ? (N + 4) * 16 : 0},
-      {(void **)&tf->q_rows,
-       cfg->mode == TPC_MODE_PRUNED ? (size_t)tf->tile_cap * kPruneRegionRows * sizeof(PruneRow) : 0},
+      {(void **)&tf->q_rec,
+       cfg->mode == TPC_MODE_PRUNED ? (size_t)tf->tile_cap * kPruneRegionRows * sizeof(PruneRec) : 0},
       {(void **)&tf->q_count, cfg->mode == TPC_MODE_PRUNED ? (size_t)tf->tile_cap * 4 : 0},
       {(void **)&tf->rr_feat,
        cfg->mode == TPC_MODE_PRUNED ? (size_t)tf->tile_cap * kPruneRegionRows * kMlpIn * 4 : 0},
       {(void **)&tf->rr_logit, cfg->mode == TPC_MODE_PRUNED ? (size_t)tf->tile_cap * kPruneRegionRows * 4 : 0},
       {(void **)&tf->rr_meta, cfg->mode == TPC_MODE_PRUNED ? (size_t)tf->tile_cap * kPruneRegionRows * 16 : 0},
       {(void **)&tf->rr_cost, cfg->mode == TPC_MODE_PRUNED ? (size_t)tf->tile_cap * kPruneRegionRows * 8 : 0},
-      {(void **)&tf->rr_tbase, cfg->mode == TPC_MODE_PRUNED ? (size_t)tf->tile_cap * 4 : 0},
       {(void **)&tf->f_params, fol ? TL * 5 * 4 : 0},
       {(void **)&tf->f_cov, fol ? TL * 15 * 4 : 0},
       {(void **)&tf->f_tref, fol ? TL * 4 : 0},
@@ -469,7 +467,7 @@ static void fill_args(tpc_tf *tf, uint32_t n, const tpc_tracks *out, Args &a) {
   a.amb_cap = tf->amb ? tf->N + 4 : 0;
   a.mlp = tf->mlp;
   a.logit_tau = tf->logit_tau;
-  a.q_rows = tf->q_rows;
+  a.q_rec = tf->q_rec;
   a.q_count = tf->q_count;
   if (tf->cfg.follow) {
     a.fl.params = tf->f_params;
@@ -549,7 +547,7 @@ static int enqueue_linking(tpc_tf *tf, const tpc_clusters *cl, Args &a, cudaStre
   stage(tf, st, "neighbours");
   tf->launches += 4;
   if (prune) {
-    launch_region_rescore(a, tf->mlp, tf->mlp_head, tf->rr_feat, tf->rr_meta, tf->rr_cost, tf->rr_logit, tf->rr_tbase,
+    launch_region_rescore(a, tf->mlp, tf->mlp_head, tf->rr_feat, tf->rr_meta, tf->rr_cost, tf->rr_logit,
                           tf->logit_tau, tf->sms, tf->cfg.mlp_engine, st);
     stage(tf, st, "prune_tiles");
     launch_prune(a, tf->mlp, tf->logit_tau, tf->sms, st);

@@ -7,11 +7,10 @@
 // scores each of them; the pair kept is the smallest (cost, j, k) among those
 // whose score sigmoid(logit) reaches tau, or the plain choice when none does.
 // Only ~2 % of clusters are ambiguous at Pb-Pb-like densities.  The neighbour
-// kernel writes the pairs of a tile's ambiguous clusters into the tile's own
-// region (i, j, k, candidate counts, quantised coordinates); k_region_feat packs
-// the regions' rows into a dense array of feature rows, the dense scorer (tcgen05
-// or mma.sync) scores it, and k_region_decide decides each cluster from its
-// contiguous rows.  Clusters that the neighbour kernel could not put in a region
+// kernel writes a tile's ambiguous clusters into the tile's own region (their
+// candidates as two masks); k_region_feat enumerates their pairs into a dense
+// array of feature rows, the dense scorer (tcgen05 or mma.sync) scores it, and
+// k_region_decide decides each cluster from its contiguous rows.  Clusters that the neighbour kernel could not put in a region
 // (windows too large to stage, or the region full) are listed instead, and
 // k_prune rescores those: each warp takes 32 listed clusters and re-enumerates
 // their pairs from global memory.
@@ -646,71 +645,112 @@ __global__ void __launch_bounds__(256) k_mlp_extract(Args a, float *__restrict__
 }
 
 // ------------------------------------------------------------------ launchers
-// ---- region rescoring in three passes.  (1) k_region_feat packs the rows of the
-// tile regions into one dense array of feature rows: a CTA step takes 32 regions,
-// takes their place in the array with one atomic (regions land in any order, each
-// stays contiguous) and records each region's first row in tbase; every thread
-// computes the 12 features of its rows.  (2) The dense scorer of either engine
-// scores the array at full tensor-core occupancy, reading the row count from the
-// device.  (3) k_region_decide gives each dense row one thread; the thread holding
-// a cluster's first row (a cluster's rows are contiguous, and never span two
-// regions) keeps the smallest (cost, j, k) among the cluster's rows whose logit
-// passes.  Each row's (cluster, j, k) and cost go to meta and cost in pass (1).
-// One kernel that ran the three phases per CTA, as a chain of 256-row batches,
-// was bound by that chain's latency (0.125-0.14 ms on the 10 ms frame against
-// 0.099 ms for the three passes with the tcgen05 scorer).
-constexpr int kRegionGroup = 32;  // regions per CTA step of k_region_feat
-__global__ void __launch_bounds__(256) k_region_feat(Args a, float *__restrict__ feat, int4 *__restrict__ meta,
-                                                     int64_t *__restrict__ cost, uint32_t *__restrict__ tbase) {
-  __shared__ int s_off[kRegionGroup + 1];
+// ---- region rescoring in three passes.  (1) k_region_feat enumerates the pairs of
+// the tile regions' records into one dense array of feature rows: a CTA step takes
+// kRegionGroup regions and their place in the array with one atomic (regions land
+// in any order, each stays contiguous) and a record per thread; then every candidate
+// pair of those records takes one thread, which loads its three clusters together
+// and, under the cut, writes the pair's 12 features to the record's next row.  (2)
+// The dense scorer of either engine scores the array at full tensor-core occupancy,
+// reading the row count from the device.  (3) k_region_decide gives each dense row
+// one thread; the thread holding a cluster's first row (a cluster's rows are
+// contiguous, in any order, and never span two regions) keeps the smallest (cost,
+// j, k) among the cluster's rows whose logit passes.  Each row's (cluster, j, k)
+// and cost go to meta and cost in pass (1).
+// Pass (1) is bound by its few dependent loads and the features' instructions.  On
+// the 10 ms frame (1.3 M rows of 0.6 M clusters) it takes 0.08 ms, 0.05 more than
+// copying rows that the neighbour kernel has written out, and saves 0.16 ms there.
+// Measured beside it: a thread per record 0.10 ms; a warp per tile, its pairs spread
+// over the lanes by shuffles, 0.13; a thread per row, which finds its pair in a third
+// mask, 0.06, but the neighbour kernel then takes 0.035 longer to fill that mask.
+// One kernel that ran the three passes per CTA, as a chain of 256-row batches, was
+// bound by that chain's latency.
+constexpr int kRegionGroup = 8;  // regions per CTA step of k_region_feat (16: 0.02 ms more on a 5 M batch)
+constexpr int kRegionThreads = 256;
+constexpr int kRegionCtasPerSm = 6;  // 40 registers (4 or 5: 0.02, 0.01 ms more)
+
+// position (from the top) of the n-th set bit of m
+__device__ __forceinline__ int nth_from_top(uint32_t m, int n) {
+  for (; n > 0; --n) m &= 0x7fffffffu >> __clz((int)m);
+  return __clz((int)m);
+}
+
+__global__ void __launch_bounds__(kRegionThreads, kRegionCtasPerSm)
+    k_region_feat(Args a, float *__restrict__ feat, int4 *__restrict__ meta, int64_t *__restrict__ cost) {
+  __shared__ int s_rec[kRegionGroup + 1], s_row[kRegionGroup];
   __shared__ uint32_t s_base;
+  __shared__ uint32_t s_warp[kRegionThreads / 32];
+  __shared__ int4 s_h[kRegionThreads], s_m[kRegionThreads];  // (i, j0, k0, next row), (mj, mk, cn, row)
+  __shared__ uint32_t s_off[kRegionThreads];                 // first candidate pair of each record
   const int tid = threadIdx.x, lane = tid & 31;
   const uint32_t ntiles = min(a.ctr[kCtrTiles], a.tile_cap);
   for (uint32_t g0 = blockIdx.x * kRegionGroup; g0 < ntiles; g0 += gridDim.x * kRegionGroup) {
     const int nreg = (int)min((uint32_t)kRegionGroup, ntiles - g0);
-    if (tid < 32) {  // the regions' row counts, their offsets and the step's place in the array
-      int c = lane < nreg ? min(a.q_count[g0 + lane], kPruneRegionRows) : 0;
-      if (c < 2) c = 0;
-      int x = c;
+    if (tid < 32) {  // the regions' records and rows, their offsets and the step's place in the array
+      const uint32_t q = lane < nreg ? (uint32_t)a.q_count[g0 + lane] : 0u;
+      const int nrec = min((int)(q >> 16), kPruneRegionRows), nrow = min((int)(q & 0xffffu), kPruneRegionRows);
+      int x = nrec, y = nrow;
       for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
+        const int xx = __shfl_up_sync(0xffffffffu, x, o), yy = __shfl_up_sync(0xffffffffu, y, o);
+        if (lane >= o) {
+          x += xx;
+          y += yy;
+        }
       }
-      uint32_t base = 0;
-      if (lane == 31 && x > 0) base = atomicAdd(&a.ctr[kCtrRegionRows], (uint32_t)x);
-      base = __shfl_sync(0xffffffffu, base, 31);
-      if (lane < nreg) tbase[g0 + lane] = base + (uint32_t)(x - c);
-      s_off[lane + 1] = x;
-      if (lane == 0) {
-        s_off[0] = 0;
-        s_base = base;
+      if (lane < kRegionGroup) {
+        s_rec[lane + 1] = x;
+        s_row[lane] = y - nrow;
       }
+      if (lane == 0) s_rec[0] = 0;
+      if (lane == 31) s_base = y > 0 ? atomicAdd(&a.ctr[kCtrRegionRows], (uint32_t)y) : 0u;
     }
     __syncthreads();
-    const int total = s_off[kRegionGroup];
-    const uint32_t base = s_base;
-    for (int gr = tid; gr < total; gr += blockDim.x) {
-      int g = 0;  // the region of row gr: the last g with s_off[g] <= gr
+    const int total = s_rec[kRegionGroup];
+    for (int e0 = 0; e0 < total; e0 += kRegionThreads) {
+      const int e = e0 + tid;
+      uint32_t pairs = 0;
+      if (e < total) {
+        int g = 0;  // the region of record e: the last g with s_rec[g] <= e
 #pragma unroll
-      for (int st = 16; st > 0; st >>= 1)
-        if (s_off[g + st] <= gr) g += st;
-      const uint32_t tile = g0 + (uint32_t)g;
-      const int4 *pr = reinterpret_cast<const int4 *>(a.q_rows + (size_t)tile * kPruneRegionRows + (gr - s_off[g]));
-      const int4 q = pr[0], c1 = pr[1], c2 = pr[2];  // (i, j, k, cn), (ti, yi, tj, yj), (tk, yk, -, -)
-      const int r = a.tile_win[2 * tile].x % kNRows;
-      const int64_t c = triplet_cost(c1.w - c1.y, c2.y - c1.y, c1.z - c1.x, c2.x - c1.x);
-      float f[kMlpIn];
-      triplet_features(r, c1.w, c1.y, c2.y, c1.z, c1.x, c2.x, c, q.w & 0xffff, (int)((unsigned)q.w >> 16), a.cost_max,
-                       f);
-      const size_t d = base + (uint32_t)gr;
-      float4 *dst = reinterpret_cast<float4 *>(feat + d * kMlpIn);
-      dst[0] = make_float4(f[0], f[1], f[2], f[3]);
-      dst[1] = make_float4(f[4], f[5], f[6], f[7]);
-      dst[2] = make_float4(f[8], f[9], f[10], f[11]);
-      meta[d] = make_int4(q.x, q.y, q.z, 0);
-      cost[d] = c;
+        for (int st = kRegionGroup / 2; st > 0; st >>= 1)
+          if (s_rec[g + st] <= e) g += st;
+        const uint32_t tile = g0 + (uint32_t)g;
+        const int4 *rec = reinterpret_cast<const int4 *>(a.q_rec + (size_t)tile * kPruneRegionRows + (e - s_rec[g]));
+        int4 h = rec[0], m = rec[1];
+        m.w = a.tile_win[2 * tile].x % kNRows;
+        h.w = (int)(s_base + (uint32_t)(s_row[g] + (h.w & 0xffff)));
+        s_h[tid] = h;
+        s_m[tid] = m;
+        pairs = (uint32_t)(__popc((uint32_t)m.x) * __popc((uint32_t)m.y));
+      }
+      uint32_t all;
+      s_off[tid] = block_exclusive_scan<kRegionThreads>(pairs, s_warp, &all);
+      __syncthreads();
+      for (uint32_t c = (uint32_t)tid; c < all; c += kRegionThreads) {
+        int o = 0;  // the record of pair c: the last o with s_off[o] <= c
+#pragma unroll
+        for (int st = kRegionThreads / 2; st > 0; st >>= 1)
+          if (s_off[o + st] <= c) o += st;
+        const int4 h = s_h[o], m = s_m[o];
+        const int v = (int)(c - s_off[o]), nk = __popc((uint32_t)m.y), x = v / nk;
+        const int j = h.y + nth_from_top((uint32_t)m.x, x), k = h.z + nth_from_top((uint32_t)m.y, v - x * nk);
+        const int2 ci = a.tq[h.x], ej = a.tq[j], ek = a.tq[k];
+        const int64_t cst = triplet_cost(ej.y - ci.y, ek.y - ci.y, ej.x - ci.x, ek.x - ci.x);
+        if (cst > a.cost_max) continue;
+        const size_t d = (uint32_t)atomicAdd(&s_h[o].w, 1);
+        float f[kMlpIn];
+        triplet_features(m.w, ej.y, ci.y, ek.y, ej.x, ci.x, ek.x, cst, m.z & 0xffff, (int)((uint32_t)m.z >> 16),
+                         a.cost_max, f);
+        float4 *dst = reinterpret_cast<float4 *>(feat + d * kMlpIn);
+        dst[0] = make_float4(f[0], f[1], f[2], f[3]);
+        dst[1] = make_float4(f[4], f[5], f[6], f[7]);
+        dst[2] = make_float4(f[8], f[9], f[10], f[11]);
+        meta[d] = make_int4(h.x, j, k, 0);
+        cost[d] = cst;
+      }
+      __syncthreads();  // the tables are rewritten by the next records
     }
-    __syncthreads();  // s_off is rewritten by the next step
+    __syncthreads();
   }
 }
 
@@ -744,10 +784,10 @@ __global__ void __launch_bounds__(256) k_region_decide(Args a, const float *__re
 
 size_t mlp_score_tc_smem();
 void launch_region_rescore(const Args &a, const MlpW *w, const MlpHead &head, float *feat, int4 *meta,
-                           int64_t *cost, float *logit, uint32_t *tbase, float logit_tau, int sms, int engine,
+                           int64_t *cost, float *logit, float logit_tau, int sms, int engine,
                            cudaStream_t st) {
   const uint32_t rows_cap = a.tile_cap * (uint32_t)kPruneRegionRows;
-  k_region_feat<<<sms * 8, 256, 0, st>>>(a, feat, meta, cost, tbase);
+  k_region_feat<<<sms * 2 * kRegionCtasPerSm, kRegionThreads, 0, st>>>(a, feat, meta, cost);
   const uint32_t *m_dev = a.ctr + kCtrRegionRows;
   if (engine == TPC_MMA_SYNC)
     k_mlp_score<<<sms * 8, kPruneWarps * 32, 0, st>>>(w, feat, rows_cap, m_dev, logit);

@@ -16,12 +16,18 @@
 // wt of the tile's time span (binary searches, all tiles in parallel).  The
 // neighbour kernel gives each tile one CTA: the bulk-copy (TMA) engine copies the
 // tile and both windows from the quantised array into shared memory, completion
-// on an mbarrier; each thread then links a contiguous run of clusters, moving its
-// window pointers forward only.  Its scans of the two windows only collect
-// candidates (indices in a 16-bit shift register); the pairs are scored after
-// both scans, so that lanes with longer windows do not drag the pair arithmetic
-// through every iteration.  Windows larger than the staging buffers are read
-// from global memory with the same arithmetic.
+// on an mbarrier; then each warp links 32 consecutive clusters at a time, a cluster
+// per lane.  Windows larger than the staging buffers are read from global memory
+// with the same arithmetic.
+//
+// What bounds it: instruction issue (82 % of the slots) and the integer pipe, which
+// takes half of them at half rate; DRAM traffic is 14 of the 16 bytes a cluster
+// needs, at a tenth of the bandwidth.  Warp instructions per 32 clusters (16.8 M
+// clusters, plain): staging 45, searches 66, scan 150, scoring and output 165.  In an
+// earlier form each thread linked a run of two clusters (a search by galloping,
+// pointers moved forward, divergent scans that pushed candidates into 16-bit shift
+// registers): 700.  Stage times, earlier -> now: 0.71 -> 0.43 ms plain and 0.81 -> 0.48
+// ms pruned on the 10 ms frame (32 M clusters), 0.154 -> 0.092 ms plain on 2 ms.
 #include "mlp_dev.cuh"
 #include "tpc_dev.cuh"
 #include "tpc_internal.h"
@@ -30,18 +36,20 @@ namespace tpc {
 
 namespace {
 
-constexpr int kMaxCand = 4;  // candidates per neighbour row kept in registers
+constexpr int kMaxCand = 4;  // candidates per neighbour row kept in registers (windows read from global memory)
 
-// Pruned mode: the pairs under the cut of the tile's ambiguous clusters (the
-// first four kept in registers while the pairs are scored, more enumerated again)
-// are written to the tile's own region of kPruneRegionRows rows (a shared-memory
-// counter reserves them, so no global atomic is taken); the rescoring kernel
-// reads the region.  Clusters with more than kPruneMaxPairs such pairs, or that
-// do not fit, go to the global list.
+// Pruned mode: the tile's ambiguous clusters (two pairs or more under the cut) go
+// to the tile's own region: for each one its candidates as two masks, and the place
+// of its pairs among the region's kPruneRegionRows rows (a shared-memory counter
+// reserves both, so no global atomic is taken); the rescoring enumerates the pairs.
+// (Written out here as 48-byte rows they cost 160 warp instructions per 32 clusters,
+// as masks 70.)  Clusters with more than kPruneMaxPairs such pairs, or that do not
+// fit, go to the global list.
 constexpr int kPruneMaxPairs = 32;
 struct NbQueue {
-  int count, end;
-  unsigned warps_done;  // the last warp to finish publishes the region's row count
+  uint32_t count;       // records << 16 | rows, also of those that did not fit
+  uint32_t end;         // the count before the first that did not fit
+  unsigned warps_done;  // the last warp to finish publishes the region's count
 };
 template <bool kPrune> struct NbExtra {};
 template <> struct NbExtra<true> { NbQueue q; };
@@ -192,148 +200,186 @@ __device__ __noinline__ void link_run(const Args &a, int li0, int li1, int cnt, 
   }
 }
 
-// The same linking for staged windows (fewer than 2048 entries each), on
-// shared-memory arrays of (t, y) that end with a sentinel entry of t = INT_MAX,
-// so that no scan needs a bounds check.  The scans of both windows only collect
-// the in-window candidates (their window-local indices, up to four per row, in
-// two registers used as a shift register of 16-bit entries); the pairs are scored
-// afterwards, so that the divergent scans stay cheap.  The best pair is the
-// smallest key (cost << 22 | j << 11 | k) over the pairs of cost <= cost_max:
-// the lexicographic minimum of (cost, j, k) whatever the order of scoring.  A
-// window test is one unsigned compare: |d| <= w  <=>  (unsigned)(d + w) <= 2 w.
-// A cluster with more than four candidates in a row (0.2 % on the synthetic
-// frames) scores every pair of its windows instead.
-template <bool kPrune>
-__device__ __forceinline__ void link_run_smem(const Args &a, int li0, int li1, int cnt, const int2 *__restrict__ sc,
-                                              const int2 *__restrict__ sp, int np, const int2 *__restrict__ sn,
-                                              int nn, int wy, int wt, int64_t cost_max, int2 *out, int base_p,
-                                              int base_n, int base_c, NbQueue *q, uint32_t *pairs,
-                                              PruneRow *region) {
-  if (li0 >= li1) return;
+// The same linking for staged windows, on shared-memory arrays of (t, y).  Lane l
+// of a warp takes cluster l of 32 consecutive ones, so the lanes' windows nearly
+// coincide and the warp stays converged: a binary search of fixed depth over
+// each window (CAP entries, kNbEnd behind the last real one) finds the first
+// entry in time, then both windows are scanned together, one entry of each row
+// per step, until both have passed the window's end.  An entry inside the pad
+// window too sets a bit; the pairs of set bits are scored afterwards in (j, k)
+// order, so that a strict comparison of the cost keeps the smaller j, then the
+// smaller k, of equal costs.  |dy| <= wy is one unsigned compare:
+// (unsigned)(dy + wy) <= 2 wy.
+//
+// A cluster whose time window holds more than 31 entries of a row (dense
+// instances; a mask has 32 bits) scores each j's pairs directly, over the entries of
+// row r+1 with |d2z| <= sqrt(cost_max), found by one more binary search.
+//
+// Measured beside it: a table of time buckets per row instead of the searches (the
+// buckets' slack costs more scan steps than the searches cost: 0.123 against 0.117 ms
+// on 2 ms); 64-bit pointers (0.117 against 0.107).  Entries are addressed by their
+// 32-bit shared-memory address (as bytes), so that a step costs no 64-bit arithmetic.
+__device__ __forceinline__ uint32_t smem_addr(const void *p) {
+  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+__device__ __forceinline__ int2 lds_entry(uint32_t addr) {
+  int2 v;
+  asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
+  return v;
+}
+template <int OFF>
+__device__ __forceinline__ int lds_time(uint32_t addr) {
+  int v;
+  asm volatile("ld.shared.b32 %0, [%1 + %2];" : "=r"(v) : "r"(addr), "n"(OFF));
+  return v;
+}
+// address of the first of CAP sorted entries from e with t >= x
+template <int S>
+__device__ __forceinline__ uint32_t nb_lower_bound(uint32_t e, int x) {
+  if (lds_time<8 * (S - 1)>(e) < x) e += 8u * S;
+  if constexpr (S > 1) return nb_lower_bound<S / 2>(e, x);
+  else return e;
+}
+// both windows' lower bounds, their steps alternating
+template <int S>
+__device__ __forceinline__ void nb_lower_bounds(uint32_t &p, uint32_t &n, int x) {
+  const int tp = lds_time<8 * (S - 1)>(p), tn = lds_time<8 * (S - 1)>(n);
+  if (tp < x) p += 8u * S;
+  if (tn < x) n += 8u * S;
+  if constexpr (S > 1) nb_lower_bounds<S / 2>(p, n, x);
+}
+
+template <bool kPrune, int THREADS, int CAP>
+__device__ __forceinline__ void link_tile_smem(const Args &a, int cnt, const int2 *__restrict__ sc,
+                                               const int2 *__restrict__ sp, int np, const int2 *__restrict__ sn,
+                                               int nn, int wy, int wt, int64_t cost_max, int2 *out, int base_p,
+                                               int base_n, int base_c, NbQueue *q, PruneRec *region) {
   const uint32_t wy2 = 2u * (uint32_t)wy;
-  const uint64_t cmax = (uint64_t)cost_max;
-  const float frac = (float)li0 / (float)cnt;
-  const int t0 = sc[li0].x;
-  int jlo = gallop_lower_bound([&](int j) { return sp[j].x; }, np, t0 - wt, (int)(frac * (float)np));
-  int klo = gallop_lower_bound([&](int k) { return sn[k].x; }, nn, t0 - wt, (int)(frac * (float)nn));
-  for (int li = li0; li < li1; ++li) {
-    const int2 ci = sc[li];
-    const int32_t ti = ci.x, yi = ci.y, tlo = ti - wt, thi = ti + wt;
-    while (sp[jlo].x < tlo) ++jlo;  // the sentinel stops both advances
-    while (sn[klo].x < tlo) ++klo;
-    // candidates: newest in the low half of c01, then the high half, then c23
-    uint32_t cj01 = 0, cj23 = 0, ck01 = 0, ck23 = 0;
-    int nj = 0, nk = 0;
-    for (int j = jlo;; ++j) {
-      const int2 e = sp[j];
-      if (e.x > thi) break;
-      if ((uint32_t)(e.y - yi + wy) <= wy2) {
-        cj23 = __byte_perm(cj23, cj01, 0x1076);  // (c23 << 16) | (c01 >> 16)
-        cj01 = __byte_perm(cj01, (uint32_t)j, 0x1054);  // (c01 << 16) | j
-        ++nj;
+  const uint64_t cut = (uint64_t)cost_max + 1u;
+  const uint32_t ac = smem_addr(sc), ap = smem_addr(sp), an = smem_addr(sn);
+  for (int li = threadIdx.x; li < cnt; li += THREADS) {
+    const int2 ci = lds_entry(ac + 8u * (uint32_t)li);
+    const int32_t ti = ci.x, yi = ci.y, tlo = ti - wt, thi = ti + wt, ylo = yi - wy, yhi = yi + wy;
+    uint32_t jlo = ap, klo = an;
+    nb_lower_bounds<CAP / 2>(jlo, klo, tlo);
+    // Two entries of each row per step.  thi - t, y - ylo and yhi - y are all
+    // nonnegative for an entry inside both windows, so the sign bit of their OR is
+    // shifted into the row's mask.
+    uint32_t mj = 0, mk = 0;
+    uint32_t pj = jlo, pk = klo;
+    const uint32_t pstop = jlo + 32 * 8;
+    int tj, tk;
+    do {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int2 ej = lds_entry(pj + 8 * h), ek = lds_entry(pk + 8 * h);
+        tj = thi - ej.x;
+        tk = thi - ek.x;
+        mj = __funnelshift_l((uint32_t)(tj | (ej.y - ylo) | (yhi - ej.y)), mj, 1);
+        mk = __funnelshift_l((uint32_t)(tk | (ek.y - ylo) | (yhi - ek.y)), mk, 1);
       }
+      pj += 16;
+      pk += 16;
+    } while ((tj & tk) >= 0 && pj != pstop);
+    const bool wide = (tj & tk) >= 0;
+    {  // bit 31 - m set: entry m from jlo (klo) lies in both windows
+      const int c = 32 - (int)((pj - jlo) >> 3);
+      mj = ~mj << c;
+      mk = ~mk << c;
     }
-    if (nj > 0)
-      for (int k = klo;; ++k) {
-        const int2 e = sn[k];
-        if (e.x > thi) break;
-        if ((uint32_t)(e.y - yi + wy) <= wy2) {
-          ck23 = __byte_perm(ck23, ck01, 0x1076);
-          ck01 = __byte_perm(ck01, (uint32_t)k, 0x1054);
-          ++nk;
-        }
-      }
-    uint64_t best = ~0ull;
-    int nc = 0;
-    auto score = [&](int j, int k, int2 ej, int2 ek) {
-      const int32_t d2y = ej.y + ek.y - 2 * yi;
-      const int32_t d2z = (ej.x + ek.x - 2 * ti) * kUmPerBin;
+    uint64_t best = cut;
+    uint32_t bj = 0, bk = 0;  // its pair, as entries from jlo and klo
+    int nc = 0;  // (pruned) pairs under the cut
+    // cost of the pair with kinks (d2y, d2z); smaller than the best so far: kept
+    auto score = [&](int32_t d2y, int32_t d2z, uint32_t j, uint32_t k) {
       const uint64_t c = (uint64_t)((int64_t)d2y * d2y) + (uint64_t)((int64_t)d2z * d2z);
-      if (c <= cmax) {
-        if (kPrune) {
-          if (nc < 4) pairs[nc * 256 + threadIdx.x] = (uint32_t)j | ((uint32_t)k << 11);
-          ++nc;
-        }
-        const uint64_t key = (c << 22) | ((uint64_t)j << 11) | (uint64_t)k;
-        best = key < best ? key : best;
+      if (kPrune) nc += c < cut;
+      if (c < best) {
+        best = c;
+        bj = j;
+        bk = k;
       }
     };
-    if (nj <= 4 && nk <= 4) {
-      // the newest two candidates of each row (unused ones read entry 0 and are not taken)
-      if (nk > 0) {
-        const int ja = (int)(cj01 & 0xffffu), jb = (int)(cj01 >> 16);
-        const int ka = (int)(ck01 & 0xffffu), kb = (int)(ck01 >> 16);
-        const int2 eja = sp[ja], eka = sn[ka];
-        score(ja, ka, eja, eka);
-        if (nj > 1) score(jb, ka, sp[jb], eka);
-        if (nk > 1) {
-          const int2 ekb = sn[kb];
-          score(ja, kb, eja, ekb);
-          if (nj > 1) score(jb, kb, sp[jb], ekb);
-        }
-      }
-      {
-        if (nj > 2 || nk > 2) {  // pairs with an older candidate (positions 2, 3 from the newest)
-          auto at = [](uint32_t c01, uint32_t c23, int pos) {
-            return (int)(((pos & 2 ? c23 : c01) >> ((pos & 1) * 16)) & 0xffffu);
-          };
-          for (int x = 0; x < nj; ++x)
-            for (int z = (x < 2 ? 2 : 0); z < nk; ++z) {
-              const int j = at(cj01, cj23, x), k = at(ck01, ck23, z);
-              score(j, k, sp[j], sn[k]);
-            }
-        }
-      }
-    } else {  // crowded: every pair of the windows
-      for (int j = jlo;; ++j) {
-        const int2 ej = sp[j];
+    // the pairs of a cluster with a wide window, in (j, k) order
+    const int rz = a.cost_rmax / kUmPerBin;  // |d2z| <= sqrt(cost_max)  <=>  |tj + tk - 2 ti| <= rz
+    const uint32_t pend = ap + 8u * (uint32_t)np, nend = an + 8u * (uint32_t)nn;
+    auto wide_pairs = [&](auto f) {
+      for (uint32_t j = jlo; j < pend; j += 8) {
+        const int2 ej = lds_entry(j);
         if (ej.x > thi) break;
-        if ((uint32_t)(ej.y - yi + wy) > wy2) continue;
-        for (int k = klo;; ++k) {
-          const int2 ek = sn[k];
-          if (ek.x > thi) break;
-          if ((uint32_t)(ek.y - yi + wy) > wy2) continue;
-          score(j, k, ej, ek);
+        if ((uint32_t)(ej.y - ylo) > wy2) continue;
+        const int t2 = 2 * ti - ej.x, k1 = min(thi, t2 + rz);
+        for (uint32_t k = nb_lower_bound<CAP / 2>(an, max(tlo, t2 - rz)); k < nend; k += 8) {
+          const int2 ek = lds_entry(k);
+          if (ek.x > k1) break;
+          if ((uint32_t)(ek.y - ylo) <= wy2) f((j - jlo) >> 3, (k - klo) >> 3, ej, ek);
         }
       }
-    }
-    out[li] = best != ~0ull ? make_int2(base_p + (int)((best >> 11) & 2047u), base_n + (int)(best & 2047u))
-                            : make_int2(-1, -1);
-    if (kPrune && nc >= 2) {
-      // the pairs go to the tile's region (rows in any order: the rescoring
-      // compares (cost, j, k) explicitly); a cluster that does not fit goes to the list
-      int old = kPruneRegionRows;
-      if (nc <= kPruneMaxPairs) old = atomicAdd(&q->count, nc);
-      if (old + nc <= kPruneRegionRows) {
-        atomicMax(&q->end, old + nc);  // reservations that fit form a prefix of the region
-        const int cn = nj | (nk << 16), ci_ = base_c + li;
-        auto put = [&](int slot, uint32_t jk) {
-          const int j = (int)(jk & 2047u), k = (int)(jk >> 11);
-          const int2 ej = sp[j], ek = sn[k];
-          PruneRow &w = region[slot];
-          reinterpret_cast<int4 *>(&w)[0] = make_int4(ci_, base_p + j, base_n + k, cn);
-          reinterpret_cast<int4 *>(&w)[1] = make_int4(ti, yi, ej.x, ej.y);
-          reinterpret_cast<int4 *>(&w)[2] = make_int4(ek.x, ek.y, 0, 0);
-        };
-        if (nc <= 4) {
-          for (int e = 0; e < nc; ++e) put(old + e, pairs[e * 256 + threadIdx.x]);
-        } else {  // more than four pairs (rare): enumerate them again from the windows
-          int slot = old;
-          for (int j = jlo;; ++j) {
-            const int2 ej = sp[j];
-            if (ej.x > thi) break;
-            if ((uint32_t)(ej.y - yi + wy) > wy2) continue;
-            for (int k = klo;; ++k) {
-              const int2 ek = sn[k];
-              if (ek.x > thi) break;
-              if ((uint32_t)(ek.y - yi + wy) > wy2) continue;
-              if ((uint64_t)triplet_cost(ej.y - yi, ek.y - yi, ej.x - ti, ek.x - ti) <= cmax)
-                put(slot++, (uint32_t)j | ((uint32_t)k << 11));
-            }
+    };
+    // the first entry of a mask; the mask without it
+    auto first = [](uint32_t m) { return (uint32_t)__clz((int)m); };
+    auto rest = [](uint32_t m, uint32_t z) { return m & (0x7fffffffu >> z); };
+    if (!wide) {
+      if (mj != 0 && mk != 0) {
+        // the first two candidates of row r+1 stay in registers over the j loop
+        const uint32_t z0 = first(mk), mk1 = rest(mk, z0);
+        const uint32_t z1 = mk1 ? first(mk1) : z0, mk2 = rest(mk1, z1);
+        const int2 e0 = lds_entry(klo + 8u * z0), e1 = lds_entry(klo + 8u * z1);
+        const int32_t y0 = e0.y - yi, x0 = (e0.x - ti) * kUmPerBin;
+        const int32_t y1 = e1.y - yi, x1 = (e1.x - ti) * kUmPerBin;
+        uint32_t m = mj;
+        do {
+          const uint32_t x = first(m);
+          m = rest(m, x);
+          const int2 ej = lds_entry(jlo + 8u * x);
+          const int32_t dy = ej.y - yi, dz = (ej.x - ti) * kUmPerBin;
+          score(dy + y0, dz + x0, x, z0);
+          if (!kPrune || mk1) score(dy + y1, dz + x1, x, z1);  // (plain: a repeated pair changes nothing)
+          for (uint32_t r = mk2, z; r; r = rest(r, z)) {
+            z = first(r);
+            const int2 ek = lds_entry(klo + 8u * z);
+            score(dy + ek.y - yi, dz + (ek.x - ti) * kUmPerBin, x, z);
           }
+        } while (m);
+      }
+    } else {
+      wide_pairs([&](uint32_t j, uint32_t k, int2 ej, int2 ek) {
+        score(ej.y + ek.y - 2 * yi, (ej.x + ek.x - 2 * ti) * kUmPerBin, j, k);
+      });
+    }
+    const int j0 = base_p + (int)((jlo - ap) >> 3), k0 = base_n + (int)((klo - an) >> 3);
+    out[li] = best < cut ? make_int2(j0 + (int)bj, k0 + (int)bk) : make_int2(-1, -1);
+    if (kPrune && nc >= 2) {
+      // The tile's region takes the cluster's masks; its pairs get the rows behind
+      // those of the clusters before it.  A wide cluster takes a record for each pair,
+      // so that the rescoring never scans a window.  The count holds
+      // (records, rows), and reservations that fit form a prefix of it; a cluster
+      // that does not fit goes to the list.
+      uint32_t old = kPruneRegionRows;
+      if (nc <= kPruneMaxPairs) old = atomicAdd(&q->count, ((wide ? (uint32_t)nc : 1u) << 16) + (uint32_t)nc);
+      int row = (int)(old & 0xffffu);
+      if (row + nc <= kPruneRegionRows) {
+        int4 *rec = reinterpret_cast<int4 *>(region + (old >> 16));
+        int nj = __popc(mj), nk = __popc(mk);
+        if (!wide) {
+          rec[0] = make_int4(base_c + li, j0, k0, row | (nc << 16));
+          rec[1] = make_int4((int)mj, (int)mk, nj | (nk << 16), 0);
+        } else {
+          nj = nk = 0;
+          int2 e;
+          for (uint32_t j = jlo; j < pend && (e = lds_entry(j)).x <= thi; j += 8) nj += (uint32_t)(e.y - ylo) <= wy2;
+          for (uint32_t k = klo; k < nend && (e = lds_entry(k)).x <= thi; k += 8) nk += (uint32_t)(e.y - ylo) <= wy2;
+          const int one = (int)0x80000000u;
+          wide_pairs([&](uint32_t j, uint32_t k, int2 ej, int2 ek) {
+            if ((uint64_t)triplet_cost(ej.y - yi, ek.y - yi, ej.x - ti, ek.x - ti) >= cut) return;
+            rec[0] = make_int4(base_c + li, j0 + (int)j, k0 + (int)k, row++ | (1 << 16));
+            rec[1] = make_int4(one, one, nj | (nk << 16), 0);
+            rec += 2;
+          });
         }
       } else {
-        amb_push(a, make_int4(base_c + li, base_p + jlo, base_n + klo, nc));
+        if (nc <= kPruneMaxPairs && row <= kPruneRegionRows) q->end = old;  // the first that does not fit
+        amb_push(a, make_int4(base_c + li, j0, k0, nc));
       }
     }
   }
@@ -344,9 +390,6 @@ __device__ __forceinline__ void link_run_smem(const Args &a, int li0, int li1, i
 // shared memory by the bulk-copy (TMA) engine: cp.async.bulk with completion on
 // an mbarrier, in 16-byte granules (two 8-byte entries), so a range [lo, hi) is
 // copied from lo & ~1 to (hi + 1) & ~1 (the array is padded past n).
-__device__ __forceinline__ uint32_t smem_addr(const void *p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
 __device__ __forceinline__ void mbar_init1(uint64_t *bar) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -371,16 +414,17 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
                : "memory");
 }
 
-template <bool kPrune> struct NbPairs {};
-template <> struct NbPairs<true> { uint32_t v[4 * 256]; };  // a thread's first four pairs under the cut
-
 // shared memory of one neighbour CTA: the quantised tile and windows, each with
-// a granule offset of 0 or 1 entry in front and a sentinel behind
-template <int TILE, int WIN>
+// a granule offset of 0 or 1 entry in front.  A window holds at most CAP - 1
+// entries; kNbEnd behind them up to CAP (the searches' depth) and for the
+// 32 steps a scan may go on.
+constexpr int kNbPad = 32;
+constexpr int kNbEnd = 1 << 30;  // later than any cluster, and far from overflow
+template <int TILE, int CAP>
 struct __align__(16) NbSmem {
   int2 c[TILE + 2];
-  int2 p[WIN + 4];
-  int2 n[WIN + 4];
+  int2 p[CAP + 2 + kNbPad];
+  int2 n[CAP + 2 + kNbPad];
   uint64_t bar;
 };
 
@@ -436,22 +480,22 @@ __device__ __forceinline__ void stage_tile_windows(const Args &a, uint32_t bid, 
 
 // ------------------------------------------------------------ neighbours
 // One CTA per tile: one thread issues the bulk copies of the tile and its two
-// windows, every thread waits on the mbarrier (bounded), one thread writes the
-// windows' sentinels, and each thread links a contiguous run of clusters.  32
-// registers per thread in plain mode, so that 8 CTAs of 256 threads share an SM
-// and hide each other's copies and uneven tiles; 40 in pruned mode (6 CTAs),
-// where the region bookkeeping spills at 32 (a persistent, double-buffered form
-// with 4-6 CTAs per SM measured 35-45 % slower: its per-tile barrier holds every
-// warp until the tile's slowest one).
+// windows, every thread waits on the mbarrier (bounded) and writes its share of the
+// entries behind the windows, then the warps link.  CTAs of 128 threads (4 or 6
+// passes of 32 clusters per warp spread the per-warp cost of the staging over more
+// clusters than the 2 or 3 of 256 threads: 0.100 -> 0.092 ms on 2 ms, 0.66 -> 0.48
+// pruned on 10 ms with the region records), 9 or 10 of them per SM by shared memory,
+// which leaves 48 registers a thread; the 1024-cluster tile's 41 KB take 256 threads.
+// (A persistent, double-buffered form of an earlier version measured 35-45 % slower:
+// its per-tile barrier holds every warp until the tile's slowest one.)
 // The work of one tile (t < the number of tiles).  `phase` is the parity of the
 // CTA's mbarrier phase to wait for; `init` is set until the CTA has initialised
 // its mbarrier (edge-row tiles do not use it).
-template <bool kPrune, int TILE, int WIN, int THREADS>
+template <bool kPrune, int TILE, int CAP, int THREADS>
 __device__ __forceinline__ void nb_tile(const Args &a, int win_cap, uint32_t t, uint32_t &phase, bool &init) {
-  static_assert(WIN < 2048 && TILE % THREADS == 0 && THREADS <= 256, "window indices are packed in 11 bits");
-  __shared__ NbSmem<TILE, WIN> sm;
+  static_assert((CAP & (CAP - 1)) == 0 && THREADS % 32 == 0, "the searches halve CAP");
+  __shared__ NbSmem<TILE, CAP> sm;
   __shared__ NbExtra<kPrune> ex;
-  __shared__ NbPairs<kPrune> pr;
   const int4 h = a.tile_win[2 * t], w = a.tile_win[2 * t + 1];
   const int key = h.x, ta = h.y, cnt = h.z - h.y;
   const int r = key % kNRows;
@@ -498,9 +542,10 @@ __device__ __forceinline__ void nb_tile(const Args &a, int win_cap, uint32_t t, 
   }
   const int2 *sc = sm.c + (ta - c0);
   int2 *s_p = sm.p + (w.x - p0), *s_n = sm.n + (w.z - n0);
-  if (ok && tid == 0 && staged) {
-    s_p[np] = make_int2(INT_MAX, 0);  // sentinels
-    s_n[nn] = make_int2(INT_MAX, 0);
+  if (ok && staged) {  // behind the windows (the copies are done)
+    const int2 end = make_int2(kNbEnd, 0);
+    for (int e = np + tid; e < CAP + kNbPad; e += THREADS) s_p[e] = end;
+    for (int e = nn + tid; e < CAP + kNbPad; e += THREADS) s_n[e] = end;
   }
   if (__syncthreads_or(!ok)) {
     if (tid == 0) raise(a.ctr, kErrTimeout);
@@ -509,50 +554,51 @@ __device__ __forceinline__ void nb_tile(const Args &a, int win_cap, uint32_t t, 
       }
     return;
   }
-  const int K = (cnt + NT - 1) / NT, li0 = tid * K, li1 = min(cnt, li0 + K);
   if (staged) {
-    uint32_t *pairs = nullptr;
-    if constexpr (kPrune) pairs = pr.v;
-    link_run_smem<kPrune>(a, li0, li1, cnt, sc, s_p, np, s_n, nn, a.wy, a.wt, a.cost_max, a.link + ta, w.x, w.z, ta,
-                          q, pairs, a.q_rows + (size_t)t * kPruneRegionRows);
+    link_tile_smem<kPrune, THREADS, CAP>(a, cnt, sc, s_p, np, s_n, nn, a.wy, a.wt, a.cost_max, a.link + ta, w.x, w.z,
+                                         ta, q, a.q_rec + (size_t)t * kPruneRegionRows);
   } else {
     const int2 *tq = a.tq;
     const int pb = w.x, nb = w.z;
+    const int K = (cnt + NT - 1) / NT, li0 = tid * K, li1 = min(cnt, li0 + K);
     link_run<kPrune>(
         a, li0, li1, cnt, [&](int i) { return sc[i]; }, [&](int j) { return tq[pb + j]; }, np,
         [&](int k) { return tq[nb + k]; }, nn, a.wy, a.wt, a.cost_max, a.link + ta, w.x, w.z, ta);
   }
-  if constexpr (kPrune) {  // rows used in this tile's region, published by the last warp to finish
+  if constexpr (kPrune) {  // records and rows of this tile's region, published by the last warp to finish
     __syncwarp();
     if ((tid & 31) == 0) {
       __threadfence_block();
-      if (atomicAdd(&q->warps_done, 1u) == (unsigned)(THREADS / 32 - 1)) a.q_count[t] = atomicAdd(&q->end, 0);
+      if (atomicAdd(&q->warps_done, 1u) == (unsigned)(THREADS / 32 - 1)) {
+        const uint32_t c = atomicAdd(&q->count, 0u);
+        a.q_count[t] = (int32_t)((c & 0xffffu) <= kPruneRegionRows ? c : atomicAdd(&q->end, 0u));
+      }
     }
   }
 }
 
 #ifndef TPC_STAGES_ONLY
-template <bool kPrune, int TILE, int WIN, int THREADS>
-__global__ void __launch_bounds__(THREADS, kPrune ? 1536 / THREADS : 2048 / THREADS)
+template <bool kPrune, int TILE, int CAP, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 128 ? 10 : 5)
     k_neighbours(Args a, int win_cap) {
   const uint32_t t = blockIdx.x;
   if (t >= min(a.ctr[kCtrTiles], a.tile_cap)) return;
   uint32_t phase = 0;
   bool init = true;
-  nb_tile<kPrune, TILE, WIN, THREADS>(a, win_cap, t, phase, init);
+  nb_tile<kPrune, TILE, CAP, THREADS>(a, win_cap, t, phase, init);
 }
 #endif
 
 // all tiles t = bid, bid + nblk, ... in one CTA (the persistent kernel); a tile
 // whose copies timed out records the error and the CTA goes on (its results are
 // not valid then, and the call reports TPC_ERR_TIMEOUT)
-template <bool kPrune, int TILE, int WIN, int THREADS>
+template <bool kPrune, int TILE, int CAP, int THREADS>
 __device__ __forceinline__ void stage_neighbours(const Args &a, int win_cap, uint32_t bid, uint32_t nblk) {
   const uint32_t ntiles = min(a.ctr[kCtrTiles], a.tile_cap);
   uint32_t phase = 0;
   bool init = true;
   for (uint32_t t = bid; t < ntiles; t += nblk) {
-    nb_tile<kPrune, TILE, WIN, THREADS>(a, win_cap, t, phase, init);
+    nb_tile<kPrune, TILE, CAP, THREADS>(a, win_cap, t, phase, init);
     __syncthreads();  // the staged buffers are free for the next tile
   }
 }
@@ -612,19 +658,19 @@ void launch_tile_windows(const Args &a, cudaStream_t st) {
   k_tile_windows<<<(tiles + 255) / 256, 256, 0, st>>>(a);
 }
 
-template <int TILE, int WIN>
+template <int TILE, int CAP, int THREADS>
 static void launch_nb(const Args &a, int row_cap, cudaStream_t st, bool prune) {
-  const int cap = row_cap > 0 && row_cap < WIN ? row_cap : WIN;
+  const int cap = row_cap > 0 && row_cap < CAP - 1 ? row_cap : CAP - 1;
   const uint32_t grid = neighbour_tiles_max(a.n, a.nkeys, TILE);
-  if (prune) k_neighbours<true, TILE, WIN, kNbThreads><<<grid, kNbThreads, 0, st>>>(a, cap);
-  else k_neighbours<false, TILE, WIN, kNbThreads><<<grid, kNbThreads, 0, st>>>(a, cap);
+  if (prune) k_neighbours<true, TILE, CAP, THREADS><<<grid, THREADS, 0, st>>>(a, cap);
+  else k_neighbours<false, TILE, CAP, THREADS><<<grid, THREADS, 0, st>>>(a, cap);
 }
 
 void launch_neighbours(const Args &a, int row_cap, int sms, cudaStream_t st, bool prune) {
   (void)sms;
-  if (a.nb_tile == 512) launch_nb<512, 896>(a, row_cap, st, prune);
-  else if (a.nb_tile == 1024) launch_nb<1024, 1664>(a, row_cap, st, prune);
-  else launch_nb<768, 1280>(a, row_cap, st, prune);
+  if (a.nb_tile == 512) launch_nb<512, 1024, 128>(a, row_cap, st, prune);
+  else if (a.nb_tile == 1024) launch_nb<1024, 2048, 256>(a, row_cap, st, prune);
+  else launch_nb<768, 1024, 128>(a, row_cap, st, prune);
 }
 
 void launch_edge_claims(const Args &a, cudaStream_t st) {

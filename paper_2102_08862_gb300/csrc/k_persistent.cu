@@ -69,7 +69,7 @@ __device__ __forceinline__ bool grid_sync(uint32_t *ctr, uint32_t nblk, uint32_t
 
 // 40 registers (6 CTAs of 256 per SM): measured on the batched workload against
 // 64 (4 CTAs, 20.3 ms) and 32 (8 CTAs, 20.2 ms, the fit spills): 18.8 ms
-template <int TILE, int WIN>
+template <int TILE, int CAP>
 __global__ void __launch_bounds__(256, 6) k_track_persistent(Args a, int vec, int win_cap) {
   const uint32_t bid = blockIdx.x, nblk = gridDim.x;
   stage_quantize(a, vec, bid, nblk);
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(256, 6) k_track_persistent(Args a, int vec, in
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
   stage_tile_windows(a, bid, nblk);
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
-  stage_neighbours<false, TILE, WIN, 256>(a, win_cap, bid, nblk);
+  stage_neighbours<false, TILE, CAP, 256>(a, win_cap, bid, nblk);
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
   stage_edge_claims(a, bid, nblk);
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
@@ -93,18 +93,18 @@ __global__ void __launch_bounds__(256, 6) k_track_persistent(Args a, int vec, in
 
 int g_pers_blocks[64][3];  // [device][tile variant]: resident CTAs per SM (0: not yet known)
 
-template <int TILE, int WIN>
+template <int TILE, int CAP>
 int launch_pers(const Args &a, int sms, int dev, int v, cudaStream_t st) {
   if (g_pers_blocks[dev][v] == 0) {
     int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_track_persistent<TILE, WIN>, 256, 0) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_track_persistent<TILE, CAP>, 256, 0) != cudaSuccess ||
         b < 1)
       return -1;
     g_pers_blocks[dev][v] = b;
   }
   const bool vec = ((((uintptr_t)a.pad | (uintptr_t)a.time | (uintptr_t)a.sector | (uintptr_t)a.row) & 15) == 0);
   const uint32_t grid = (uint32_t)sms * (uint32_t)g_pers_blocks[dev][v];
-  k_track_persistent<TILE, WIN><<<grid, 256, 0, st>>>(a, vec ? 1 : 0, WIN);
+  k_track_persistent<TILE, CAP><<<grid, 256, 0, st>>>(a, vec ? 1 : 0, CAP - 1);
   return 0;
 }
 
@@ -118,18 +118,18 @@ int persistent_prepare(int dev) {
     g_pers_blocks[dev][v] = b;
     return 0;
   };
-  int rc = occ(k_track_persistent<512, 896>, 0);
-  rc |= occ(k_track_persistent<768, 1280>, 1);
-  rc |= occ(k_track_persistent<1024, 1664>, 2);
+  int rc = occ(k_track_persistent<512, 1024>, 0);
+  rc |= occ(k_track_persistent<768, 1024>, 1);
+  rc |= occ(k_track_persistent<1024, 2048>, 2);
   return rc;
 }
 
 int launch_persistent(const Args &a, int sms, cudaStream_t st) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
-  if (a.nb_tile == 512) return launch_pers<512, 896>(a, sms, dev, 0, st);
-  if (a.nb_tile == 1024) return launch_pers<1024, 1664>(a, sms, dev, 2, st);
-  return launch_pers<768, 1280>(a, sms, dev, 1, st);
+  if (a.nb_tile == 512) return launch_pers<512, 1024>(a, sms, dev, 0, st);
+  if (a.nb_tile == 1024) return launch_pers<1024, 2048>(a, sms, dev, 2, st);
+  return launch_pers<768, 1024>(a, sms, dev, 1, st);
 }
 
 }  // namespace tpc

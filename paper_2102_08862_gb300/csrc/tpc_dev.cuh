@@ -142,8 +142,8 @@ struct Args {
   uint32_t amb_cap;
   const struct MlpW *mlp;  // packed classifier weights
   float logit_tau;         // a pair is kept when its logit >= logit_tau
-  struct PruneRow *q_rows;  // per neighbour tile: kPruneRegionRows rows
-  int32_t *q_count;         // per neighbour tile: rows used in its region
+  struct PruneRec *q_rec;  // per neighbour tile: up to kPruneRegionRows records
+  int32_t *q_count;        // per neighbour tile: records << 16 | rows of its region
   // track follower (follow mode): the chain tracks' fit records, claims and joins
   struct Follow {
     const float *params, *cov, *t_ref;  // fit of the chain tracks ([track][5], [track][15], [track])
@@ -163,15 +163,17 @@ struct Args {
     int4 *xlist;        // [track_list_cap][2] tracks that leave their sector: (A, exit row, -, -), state at the exit
   } fl;
 };
-// rows of a neighbour tile's region in pruned mode
+// A neighbour tile's region in pruned mode: its ambiguous clusters (two pairs or
+// more under the cost cut each) and the rows their pairs take.
 constexpr int kPruneRegionRows = 128;
-// one pair under the cost cut of an ambiguous cluster: sorted positions of the
-// triplet, the cluster's candidate counts and the quantised (t, y) of the three
-// clusters (so that the rescoring reads no cluster arrays)
-struct __align__(16) PruneRow {
-  int32_t i, j, k, cn;  // cn = nj | nk << 16
-  int32_t ti, yi, tj, yj;
-  int32_t tk, yk, pad0, pad1;
+// An ambiguous cluster: its sorted position, the first entries of its time windows
+// in rows r-1 and r+1, the first of its rows in the region | its pairs under the
+// cut << 16, its candidates: bit 31 - m of mj (mk) is set when entry j0 + m (k0 + m)
+// lies in both windows; and its numbers of candidates nj | nk << 16.  A cluster with
+// windows of more than 32 entries has a record for each of its pairs.
+struct __align__(16) PruneRec {
+  int32_t i, j0, k0, rows;
+  uint32_t mj, mk, cn, pad;
 };
 
 __device__ __forceinline__ int32_t caller_index(const Args &a, int32_t i) { return a.perm ? a.perm[i] : i; }

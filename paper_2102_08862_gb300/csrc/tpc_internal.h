@@ -9,11 +9,9 @@ namespace tpc {
 // neighbour kernel: rows are cut into tiles of nb_tile clusters; a CTA stages its
 // tile and the matching time windows of rows r-1 and r+1 (up to the variant's
 // window capacity each, more goes through global memory).  Variants (tile,
-// window, threads): (512, 896, 256), (768, 1280, 256), (1024, 1664, 256); the
+// window + 1, threads): (512, 1024, 128), (768, 1024, 128), (1024, 2048, 256); the
 // default is 768, the autotuner may pick another.
-constexpr int kNbThreads = 256;
 constexpr int kNbTile = 768;
-constexpr int kNbWin = 1280;
 constexpr int kNbTileMin = 512;
 inline bool nb_tile_ok(int t) { return t == 512 || t == 768 || t == 1024; }
 // look-back tiles: clusters per tile of the link kernel, start hits per tile of the walk
@@ -102,12 +100,12 @@ int launch_mlp_score_tc(const MlpW *w, const MlpHead &head, const float *feat, u
                         int sms, cudaStream_t st);
 // opts the tcgen05 dense scorer in to its shared memory on the current device (0 on success)
 int mlp_score_tc_prepare();
-// pruned mode: the tile regions' rows gathered into feat (tile_cap * 128 rows of 12
-// floats; meta and cost: each row's (cluster, j, k) and cost), scored by the dense
-// scorer of the engine into logit, and their clusters decided (tbase: tile_cap
-// region offsets); three launches
+// pruned mode: the pairs of the tile regions' clusters as rows of feat (tile_cap *
+// 128 rows of 12 floats; meta and cost: each row's (cluster, j, k) and cost), scored
+// by the dense scorer of the engine into logit, and their clusters decided; three
+// launches
 void launch_region_rescore(const Args &a, const MlpW *w, const MlpHead &head, float *feat, int4 *meta,
-                           int64_t *cost, float *logit, uint32_t *tbase, float logit_tau, int sms, int engine,
+                           int64_t *cost, float *logit, float logit_tau, int sms, int engine,
                            cudaStream_t st);
 void launch_mlp_extract(const Args &a, float *feat, uint8_t *label, int32_t *tri, uint32_t cap, uint32_t *count,
                         cudaStream_t st);
