@@ -219,7 +219,7 @@ static std::vector<Part> plan_arena(tpc_tf *tf, const tpc_tf_config *cfg) {
       {(void **)&tf->tile_off, (size_t)(tf->nkeys + 1) * 4},
       {(void **)&tf->tile_win, (size_t)tf->tile_cap * 2 * 16},
       {(void **)&tf->link, (N + 4) * 8},
-      {(void **)&tf->tq, (N + 8) * 8},
+      {(void **)&tf->tq, (N + 8) * 8},  // (directly behind link: sort_record_bytes)
       {(void **)&tf->mup16, (N + 16) * 2},
       {(void **)&tf->starts, (N / 2 + 2) * 8},
       {(void **)&tf->trk_key, (size_t)(tf->track_list_cap + 1) * 4},
@@ -508,6 +508,12 @@ static void fill_args(tpc_tf *tf, uint32_t n, const tpc_tracks *out, Args &a) {
   }
 }
 
+// The sort's records live in the link and quantised-cluster arrays, neighbours in
+// the arena (plan_arena) and not yet written when it runs.
+static size_t sort_record_bytes(const tpc_tf *tf) {
+  return (size_t)(reinterpret_cast<const char *>(tf->tq + tf->N + 8) - reinterpret_cast<const char *>(tf->link));
+}
+
 // A0-A2 (with the classifier's rescoring when prune is set) on stream st.
 static int enqueue_linking(tpc_tf *tf, const tpc_clusters *cl, Args &a, cudaStream_t st, bool prune) {
   const uint32_t n = cl->n;
@@ -534,7 +540,8 @@ static int enqueue_linking(tpc_tf *tf, const tpc_clusters *cl, Args &a, cudaStre
     a.time = tf->s_time;
     a.perm = tf->perm;
     const int nl = launch_sort(a, cl->sector, cl->row, cl->pad, cl->time, tf->s_sector, tf->s_row, tf->s_pad,
-                               tf->s_time, tf->perm, tf->sort_scratch, tf->sort_scratch_bytes, tf->sms, st);
+                               tf->s_time, tf->perm, tf->sort_scratch, tf->sort_scratch_bytes, tf->link,
+                               sort_record_bytes(tf), tf->sms, st);
     if (nl < 0) return fail(TPC_ERR_CUDA, "sort of unsorted input failed");
     tf->launches += nl;
     stage(tf, st, "sort");
@@ -585,7 +592,8 @@ static int enqueue_persistent(tpc_tf *tf, const tpc_clusters *cl, Args &a, cudaS
     a.time = tf->s_time;
     a.perm = tf->perm;
     const int nl = launch_sort(a, cl->sector, cl->row, cl->pad, cl->time, tf->s_sector, tf->s_row, tf->s_pad,
-                               tf->s_time, tf->perm, tf->sort_scratch, tf->sort_scratch_bytes, tf->sms, st);
+                               tf->s_time, tf->perm, tf->sort_scratch, tf->sort_scratch_bytes, tf->link,
+                               sort_record_bytes(tf), tf->sms, st);
     if (nl < 0) return fail(TPC_ERR_CUDA, "sort of unsorted input failed");
     tf->launches += nl;
     stage(tf, st, "sort");

@@ -55,9 +55,10 @@ inline size_t follow_tiles(uint32_t n, int n_min, uint32_t track_list_cap) {
   return ((nt < track_list_cap ? nt : track_list_cap) + 255) / 256 + 1;
 }
 // unsorted input: stable sort by (sector, row, time, pad) into the sorted views
+// (records: 16 bytes per cluster, free again when the sort is done)
 int launch_sort(const Args &a, const uint16_t *sector, const uint16_t *row, const float *pad, const float *time,
                 uint16_t *s_sector, uint16_t *s_row, float *s_pad, float *s_time, int32_t *perm, void *scratch,
-                size_t scratch_bytes, int sms, cudaStream_t st);
+                size_t scratch_bytes, void *records, size_t records_bytes, int sms, cudaStream_t st);
 size_t sort_scratch_bytes(uint32_t max_n);
 // hit removal: clusters with ct >= 0 in caller order (uses a.lb_links and a.ctr,
 // which must be cleared)
