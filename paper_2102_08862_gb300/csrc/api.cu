@@ -61,7 +61,7 @@ struct tpc_tf {
   int2 *link = nullptr;
   int2 *tq = nullptr;  // quantised (t, y) of every sorted cluster
   uint16_t *mup16 = nullptr;
-  int2 *starts = nullptr;
+  char *starts = nullptr;  // start list and start mask
   int32_t *trk_key = nullptr, *trk_len = nullptr, *chain = nullptr;
   uint16_t *trk_rl = nullptr;
   uint32_t *sec_tr = nullptr;  // [2][nsect] first track id and track count of each sector
@@ -221,7 +221,7 @@ static std::vector<Part> plan_arena(tpc_tf *tf, const tpc_tf_config *cfg) {
       {(void **)&tf->link, (N + 4) * 8},
       {(void **)&tf->tq, (N + 8) * 8},  // (directly behind link: sort_record_bytes)
       {(void **)&tf->mup16, (N + 16) * 2},
-      {(void **)&tf->starts, (N / 2 + 2) * 8},
+      {(void **)&tf->starts, starts_bytes(N)},
       {(void **)&tf->trk_key, (size_t)(tf->track_list_cap + 1) * 4},
       {(void **)&tf->trk_len, (size_t)(tf->track_list_cap + 1) * 4},
       {(void **)&tf->trk_rl, (size_t)(tf->track_list_cap + 8) * 2},  // read in groups of 8
@@ -441,7 +441,8 @@ static void fill_args(tpc_tf *tf, uint32_t n, const tpc_tracks *out, Args &a) {
   a.link = tf->link;
   a.tq = tf->tq;
   a.mup16 = tf->mup16;
-  a.starts = tf->starts;
+  a.starts = reinterpret_cast<int32_t *>(tf->starts);
+  a.start_bits = reinterpret_cast<uint32_t *>(tf->starts + start_bits_offset(n));
   a.trk_key = tf->trk_key;
   a.trk_len = tf->trk_len;
   a.trk_rl = tf->trk_rl;
@@ -669,7 +670,7 @@ extern "C" int tpc_track_timeframe(tpc_tf *tf, const tpc_clusters *cl, const tpc
       const int rc = enqueue_assign_fit(tf, a, st);  // cluster_track is final after the assignment
       if (rc != TPC_OK) return rc;
     }
-    tf->launches += 4;  // links, walk, assign, fit
+    tf->launches += 4 + !links_with_list(n);  // links, start list, walk, assign, fit
   } else {
     // chains and their fit into the follower's records, then following and joining
     // (cluster_track holds the chain ids in between), then the refit of the
@@ -706,7 +707,7 @@ extern "C" int tpc_track_timeframe(tpc_tf *tf, const tpc_clusters *cl, const tpc
     launch_follow_ct(a, tf->sms, st);
     if (tf->record_ct) TPC_CK(cudaEventRecord(tf->ev_ct, st));  // cluster_track is final
     stage(tf, st, "relabel");
-    tf->launches += 9;  // links, walk, assign, fit, claim reset, time samples, follow, refit, relabel
+    tf->launches += 9 + !links_with_list(n);  // links, start list, walk, assign, fit, claim reset, time samples, follow, refit, relabel
     if (tf->cfg.follow == 2 && out->next_track && out->track_capacity > 0) {
       TPC_CK(cudaMemsetAsync(tf->f_pred_claim, 0xff, (size_t)tf->track_list_cap * 4, st));
       launch_sector_links(a, tf->sms, st);

@@ -7,11 +7,11 @@
 // mutual down link; chains of at least n_min clusters become tracks, numbered in
 // the order of their start cluster.
 //
-// GB300 design.  k_links streams the link array in 2048-cluster tiles (8
-// consecutive clusters per thread), stores each mutual up link as a 16-bit index
-// inside row r+1 (a 32M-cluster frame's links then take 64 MB and stay in L2 for
-// the walk) and compacts the start hits in cluster order with a block scan plus a
-// decoupled look-back across tiles.  k_walk gives each start hit one thread: it
+// GB300 design.  k_links streams the link array, stores each mutual up link as a
+// 16-bit index inside row r+1 (a 32M-cluster frame's links then take 64 MB and stay in
+// L2 for the walk) and marks the start hits in a bit mask; k_start_list compacts them
+// in cluster order with a block scan plus a decoupled look-back across tiles.  k_walk
+// gives each start hit one thread: it
 // follows the chain n_min - 1 links to decide whether it is a track, takes its
 // track id from a second ordered compaction, then walks the whole chain writing
 // the chain's cluster positions as [step][track], so the fit reads them coalesced
@@ -30,122 +30,130 @@ namespace tpc {
 
 namespace {
 constexpr int kThreads = 256;
-constexpr int kItems = kLinkTileN / 256;         // consecutive clusters per thread in k_links
-constexpr int kLinkTile = kThreads * kItems;     // clusters per look-back tile
+constexpr int kItems = kLinkTileN / kThreads;    // clusters per thread of a hit-removal tile
+constexpr int kLinkTile = kThreads * kItems;     // clusters per look-back tile of the hit removal
 constexpr uint16_t kNone16 = 0xffff;
 
-// last key with rb[key] <= i
-__device__ __forceinline__ int key_of(const int32_t *rb, int i, int nkeys) {
-  int lo = 0, hi = nkeys;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (rb[mid] <= i) lo = mid; else hi = mid;
-  }
-  return lo;
-}
 }  // namespace
 
-// A2 + A3: mup[i] = up[i] if down[up[i]] = i; start(i) = no mutual down, a mutual up.
-// The row table rb (row_begin) sits in shared memory for up to 36 sectors and is
-// read through the L1 cache for batched calls with more.
-// THREADS threads of a CTA take a 2048-cluster tile, kLinkTileN / THREADS consecutive
-// clusters each (8 for the persistent kernel's 256 threads, 4 for k_links' 512).
-template <bool kSmemRb, int THREADS>
-__device__ __forceinline__ void stage_links(const Args &a) {
-  constexpr int kItems = kLinkTileN / THREADS;
-  static_assert(kItems == 4 || kItems % 8 == 0, "the 16-bit link stores take 4 or 8 per vector");
-  __shared__ int32_t s_rb[kSmemRb ? kNKeys + 1 : 1];
-  __shared__ uint32_t s_tile, s_prefix;
-  __shared__ uint32_t s_warp[THREADS / 32];
-  const int nkeys = a.nkeys;
+// A2 + A3: mup[i] = up[i] if down[up[i]] = i; start(i) = no mutual down, a mutual up,
+// as a bit mask over the clusters.  A step of a CTA takes kLinkStep clusters; thread t
+// holds clusters t, t + 256, ... of it, so that a warp's loads, and its gathers of the
+// partners' links (the partners of neighbours in time are neighbours too), touch a few
+// lines each.  Steps share nothing and need no barrier, so that the dependent loads
+// (link, partners' links) of 64 warps overlap.
+// What bounds it: the latency of those two loads and the instructions between them (58
+// % of the issue slots); 2.6 TB/s of DRAM traffic.  An earlier form gave a thread 8
+// consecutive clusters (every lane of a gather met a line of its own) and compacted the
+// start hits in the same pass: 0.27 ms on the 10 ms frame, 0.061 on 2 ms.  With
+// coalesced gathers alone it took 0.25: the barriers around each tile's look-back were
+// what its warps waited for.  Now 0.125 and 0.042 with the start list.
+constexpr int kLinkItems = 4;
+constexpr int kLinkStep = kThreads * kLinkItems;
+__device__ __forceinline__ void stage_links(const Args &a, uint32_t bid, uint32_t nblk) {
   const int32_t *rb = a.row_begin;
-  if constexpr (kSmemRb) {
-    for (int k = threadIdx.x; k <= nkeys; k += THREADS) s_rb[k] = a.row_begin[k];
-    rb = s_rb;
-  }
-  const uint32_t n = a.n;
-  const uint32_t n_tiles = (n + kLinkTileN - 1) / kLinkTileN;
+  const int nkeys = a.nkeys;
+  const uint32_t n = a.n, steps = (n + kLinkStep - 1) / kLinkStep;
   const uint64_t keep = l2_keep_policy();
+  const int lane = threadIdx.x & 31;
   bool bad = false;
+  for (uint32_t step = bid; step < steps; step += nblk) {
+    const int i0 = (int)(step * kLinkStep + threadIdx.x);
+    // all loads first: the thread's links, then the partner links they point to
+    int2 l[kLinkItems];
+#pragma unroll
+    for (int q = 0; q < kLinkItems; ++q)
+      l[q] = i0 + q * kThreads < (int)n ? __ldcs(a.link + i0 + q * kThreads) : make_int2(-1, -1);
+    int32_t pu[kLinkItems], pd[kLinkItems];  // up partner's down link, down partner's up link
+#pragma unroll
+    for (int q = 0; q < kLinkItems; ++q) {
+      pu[q] = l[q].y >= 0 ? a.link[l[q].y].x : -2;
+      pd[q] = l[q].x >= 0 ? a.link[l[q].x].y : -2;
+    }
+    // the key of the step's first cluster, while the loads are under way: the last one
+    // with rb[key] <= i (a warp's 32 probes per round)
+    int key = 0;
+    {
+      const int first = (int)(step * kLinkStep);
+      for (int span = nkeys; span > 1;) {
+        const int w = (span + 31) >> 5, k = key + (lane + 1) * w;
+        const int c = __popc(__ballot_sync(0xffffffffu, k < key + span && rb[min(k, nkeys)] <= first));
+        key += c * w;
+        span = min(w, span - c * w);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kLinkItems; ++q) {
+      const int i = i0 + q * kThreads;
+      uint16_t m16 = kNone16;
+      const int32_t mup = pu[q] == i ? l[q].y : -1;
+      const bool mdn = pd[q] == i;
+      if (i < (int)n) {
+        // its key, from the previous cluster's, in steps of growing size
+        for (int g = 1; key + 1 < nkeys && i >= rb[key + 1];) {
+          if (key + g < nkeys && i >= rb[key + g]) {
+            key += g;
+            g <<= 1;
+          } else {
+            g = 1;
+          }
+        }
+        if (mup >= 0) {
+          const int d = mup - rb[key + 1];
+          if (d < 0 || d >= kNone16) bad = true; else m16 = (uint16_t)d;
+        }
+        st_keep_u16(a.mup16 + i, m16, keep);
+      }
+      const uint32_t bits = __ballot_sync(0xffffffffu, i < (int)n && mup >= 0 && !mdn);
+      if (lane == 0 && i < (int)n) a.start_bits[i >> 5] = bits;
+    }
+  }
+  if (bad) raise(a.ctr, kErrRowCap);
+}
+
+// The start hits in cluster order: each thread of a tile takes kListWords words of the
+// mask (a tile is kListTileN clusters); positions come from a block scan and a
+// decoupled look-back across tiles taken in order from a counter.  The mask is 1/64 of
+// the links' bytes, so the look-back chain is short.
+constexpr int kListWords = 4;
+constexpr int kListTileN = 32 * kListWords * kThreads;
+static_assert(kListTileN >= kLinkTileN, "look-back words");
+__device__ __forceinline__ void stage_start_list(const Args &a) {
+  __shared__ uint32_t s_tile, s_prefix;
+  __shared__ uint32_t s_warp[kThreads / 32];
+  const uint32_t n = a.n, words = (n + 31) / 32, n_tiles = (n + kListTileN - 1) / kListTileN;
   for (;;) {
     if (threadIdx.x == 0) s_tile = atomicAdd(&a.ctr[kCtrTileLinks], 1u);
     __syncthreads();
     const uint32_t tile = s_tile;
     if (tile >= n_tiles) break;
-    const int i0 = (int)(tile * kLinkTileN + threadIdx.x * kItems);
-    int key = i0 < (int)n ? key_of(rb, i0, nkeys) : 0;
-    uint32_t flags = 0;
-    uint16_t m16[kItems];
-    int32_t skey[kItems];
-    // all loads first: the thread's links (8 B each, contiguous), then the
-    // partner links they point to, so that the gathers are in flight together
-    int2 l[kItems];
-    if (i0 + kItems <= (int)n) {
-#pragma unroll
-      for (int v = 0; v < kItems / 2; ++v) {
-        const int4 w = __ldcs(reinterpret_cast<const int4 *>(a.link + i0) + v);
-        l[2 * v] = make_int2(w.x, w.y);
-        l[2 * v + 1] = make_int2(w.z, w.w);
-      }
+    const uint32_t w0 = (tile * kThreads + threadIdx.x) * kListWords;
+    uint32_t bits[kListWords], count = 0, total;
+    if (w0 + kListWords <= words) {
+      const uint4 v = *reinterpret_cast<const uint4 *>(a.start_bits + w0);
+      bits[0] = v.x, bits[1] = v.y, bits[2] = v.z, bits[3] = v.w;
     } else {
 #pragma unroll
-      for (int q = 0; q < kItems; ++q) l[q] = i0 + q < (int)n ? __ldcs(a.link + i0 + q) : make_int2(-1, -1);
-    }
-    int32_t pu[kItems], pd[kItems];  // up partner's down link, down partner's up link
-#pragma unroll
-    for (int q = 0; q < kItems; ++q) {
-      pu[q] = l[q].y >= 0 ? a.link[l[q].y].x : -2;
-      pd[q] = l[q].x >= 0 ? a.link[l[q].x].y : -2;
+      for (int q = 0; q < kListWords; ++q) bits[q] = w0 + q < words ? a.start_bits[w0 + q] : 0u;
     }
 #pragma unroll
-    for (int q = 0; q < kItems; ++q) {
-      const int i = i0 + q;
-      m16[q] = kNone16;
-      skey[q] = 0;
-      if (i >= (int)n) continue;
-      while (key < nkeys - 1 && i >= rb[key + 1]) ++key;
-      const int32_t mup = pu[q] == i ? l[q].y : -1;
-      const int32_t mdn = pd[q] == i ? l[q].x : -1;
-      if (mup >= 0) {
-        const int d = mup - rb[key + 1];
-        if (d < 0 || d >= kNone16) bad = true; else m16[q] = (uint16_t)d;
-      }
-      skey[q] = key;
-      if (mdn < 0 && mup >= 0) flags |= 1u << q;
-    }
-    if (i0 + kItems <= (int)n) {
-      auto pk = [&](int q) { return (uint32_t)m16[q] | ((uint32_t)m16[q + 1] << 16); };
-      if constexpr (kItems == 4) {
-        st_keep_v2(a.mup16 + i0, make_uint2(pk(0), pk(2)), keep);
-      } else {
-#pragma unroll
-        for (int v = 0; v < kItems / 8; ++v)
-          st_keep_v4(a.mup16 + i0 + 8 * v, make_uint4(pk(8 * v), pk(8 * v + 2), pk(8 * v + 4), pk(8 * v + 6)),
-                     keep);
-      }
-    } else {
-#pragma unroll
-      for (int q = 0; q < kItems; ++q)
-        if (i0 + q < (int)n) st_keep_u16(a.mup16 + i0 + q, m16[q], keep);
-    }
-    uint32_t total;
-    const uint32_t excl = block_exclusive_scan<THREADS>((uint32_t)__popc(flags), s_warp, &total);
+    for (int q = 0; q < kListWords; ++q) count += (uint32_t)__popc(bits[q]);
+    const uint32_t excl = block_exclusive_scan<kThreads>(count, s_warp, &total);
     if (threadIdx.x < 32) {
       const uint32_t pre = lookback_exclusive(a.lb_links, tile, total, a.ctr, a.spin_limit);
-      if (threadIdx.x == 0) s_prefix = pre;
+      if (threadIdx.x == 0) {
+        s_prefix = pre;
+        if (tile == n_tiles - 1) a.ctr[kCtrStarts] = pre + total;
+      }
     }
     __syncthreads();
     uint32_t pos = s_prefix + excl;
 #pragma unroll
-    for (int q = 0; q < kItems; ++q)
-      if ((flags >> q) & 1u) {
-        if (pos < a.starts_cap) a.starts[pos] = make_int2(i0 + q, skey[q]);
-        ++pos;
-      }
-    if (tile == n_tiles - 1 && threadIdx.x == 0) a.ctr[kCtrStarts] = s_prefix + total;
+    for (int q = 0; q < kListWords; ++q)
+      for (uint32_t b = bits[q]; b; b &= b - 1u, ++pos)
+        if (pos < a.starts_cap) a.starts[pos] = (int32_t)(32u * (w0 + q)) + __ffs((int)b) - 1;
     __syncthreads();
   }
-  if (bad) raise(a.ctr, kErrRowCap);
 }
 
 // A4: one start hit per thread (kWalkChains; walking two or four chains per
@@ -195,7 +203,11 @@ __device__ __forceinline__ void stage_walk(const Args &a, uint32_t bid) {
     int c[C], kk[C], len[C];
 #pragma unroll
     for (int q = 0; q < C; ++q) {
-      st[q] = j + q < ns ? a.starts[j + q] : make_int2(-1, 0);
+      st[q] = make_int2(-1, 0);
+      if (j + q < ns) {
+        const int32_t i = a.starts[j + q];
+        st[q] = make_int2(i, min((int)a.sector[i] * kNRows + (int)a.row[i], a.nkeys - 1));
+      }
       c[q] = st[q].x;
       kk[q] = st[q].y;
       len[q] = c[q] >= 0;
@@ -359,12 +371,20 @@ __device__ __forceinline__ void stage_assign(const Args &a, uint32_t bid, uint32
 }
 
 #ifndef TPC_STAGES_ONLY
-constexpr int kLinkThreads = 256;
-constexpr int kLinkCtasPerSm = 5;  // the register limit at 48 per thread: their look-back waits overlap
-template <bool kSmemRb>
-__global__ void __launch_bounds__(kLinkThreads) k_links(Args a) {
-  stage_links<kSmemRb, kLinkThreads>(a);
+// with_list: the last CTA to finish makes the start list too
+__global__ void __launch_bounds__(kThreads, 8) k_links(Args a, int with_list) {
+  stage_links(a, blockIdx.x, gridDim.x);
+  if (!with_list) return;
+  __shared__ bool s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(&a.ctr[kCtrLinksDone], 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  stage_start_list(a);
 }
+__global__ void __launch_bounds__(kThreads) k_start_list(Args a) { stage_start_list(a); }
 template <bool kSmemRb>
 __global__ void __launch_bounds__(kThreads) k_walk(Args a) {
   stage_walk<kSmemRb>(a, blockIdx.x);
@@ -488,12 +508,17 @@ __global__ void k_debug_links(Args a, int32_t *mup, uint8_t *is_start) {
   }
 }
 
+// Up to one tile of the list (32768 clusters) its own launch would cost more than the
+// list itself: 0.186 against 0.175 ms for a frame of 7600 clusters.
+bool links_with_list(uint32_t n) { return n <= (uint32_t)kListTileN; }
+
 void launch_links(const Args &a, int sms, cudaStream_t st) {
-  const uint32_t tiles = (a.n + kLinkTileN - 1) / kLinkTileN;
-  const uint32_t cap = (uint32_t)sms * (uint32_t)kLinkCtasPerSm;
-  const uint32_t grid = tiles < cap ? (tiles ? tiles : 1u) : cap;
-  if (a.nkeys <= kNKeys) k_links<true><<<grid, kLinkThreads, 0, st>>>(a);
-  else k_links<false><<<grid, kLinkThreads, 0, st>>>(a);
+  const uint32_t steps = (a.n + kLinkStep - 1) / kLinkStep, cap = (uint32_t)sms * 8u;
+  const bool with_list = links_with_list(a.n);
+  k_links<<<steps < cap ? (steps ? steps : 1u) : cap, kThreads, 0, st>>>(a, with_list ? 1 : 0);
+  if (with_list) return;
+  const uint32_t tiles = (a.n + kListTileN - 1) / kListTileN;
+  k_start_list<<<tiles < cap ? tiles : cap, kThreads, 0, st>>>(a);
 }
 
 void launch_walk(const Args &a, int sms, cudaStream_t st) {

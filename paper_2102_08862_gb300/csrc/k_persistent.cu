@@ -7,9 +7,9 @@
 // stages in one kernel, one after the other, with a grid-wide barrier between
 // stages that depend on each other: validation and quantisation together with
 // the (sector, row) keys; the tile table (one block); the tile windows; the
-// neighbours; the edge-row claims; the mutual links and start hits; the chain
-// walk; the cluster_track assignment together with the Kalman fit.  The grid is
-// as many CTAs as fit on the GPU at once, so that every CTA is resident; each
+// neighbours; the edge-row claims; the mutual links and start hits; the start
+// list; the chain walk; the cluster_track assignment together with the Kalman fit.
+// The grid is as many CTAs as fit on the GPU at once, so that every CTA is resident; each
 // barrier wait is bounded and records TPC_ERR_TIMEOUT when it gives up (another
 // kernel holding SMs would do that), after which every CTA returns.
 #define TPC_STAGES_ONLY
@@ -83,7 +83,9 @@ __global__ void __launch_bounds__(256, 6) k_track_persistent(Args a, int vec, in
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
   stage_edge_claims(a, bid, nblk);
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
-  stage_links<false, 256>(a);
+  stage_links(a, bid, nblk);
+  if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
+  stage_start_list(a);
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
   stage_walk<false>(a, bid);
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;

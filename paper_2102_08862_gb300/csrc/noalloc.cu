@@ -85,7 +85,9 @@ size_t carve(unsigned char *base, uint32_t n, uint32_t list_cap, Args *a, size_t
   a->link = reinterpret_cast<int2 *>(take(((size_t)n + 4) * 8));
   a->tq = reinterpret_cast<int2 *>(take(((size_t)n + 8) * 8));
   a->mup16 = reinterpret_cast<uint16_t *>(take(((size_t)n + 16) * 2));
-  a->starts = reinterpret_cast<int2 *>(take(((size_t)n / 2 + 2) * 8));
+  unsigned char *starts = take(starts_bytes(n));
+  a->starts = reinterpret_cast<int32_t *>(starts);
+  a->start_bits = reinterpret_cast<uint32_t *>(starts ? starts + start_bits_offset(n) : nullptr);
   a->trk_key = reinterpret_cast<int32_t *>(take(((size_t)list_cap + 1) * 4));
   a->trk_len = reinterpret_cast<int32_t *>(take(((size_t)list_cap + 1) * 4));
   a->chain = reinterpret_cast<int32_t *>(take((size_t)kNRows * list_cap * 4));

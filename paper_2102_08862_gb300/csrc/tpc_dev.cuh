@@ -82,6 +82,7 @@ enum : int {
   kCtrBarGen = 18,          // persistent kernel: grid barriers passed
   kCtrLinkList = 19,        // cross-sector links: tracks that leave their sector (searched)
   kCtrRegionRows = 20,      // pruned mode: region rows gathered for the dense rescoring
+  kCtrLinksDone = 21,       // link kernel: CTAs that have finished
   kNCounters = 22           // (even: the 8-byte look-back words follow the counters)
 };
 
@@ -108,14 +109,15 @@ struct Args {
   uint32_t tile_cap;       // tiles the arena holds
   int2 *link;              // [n] (down, up) as sorted positions, -1 = none
   uint16_t *mup16;         // [n] mutual up link as index inside row r+1, 0xffff = none
-  int2 *starts;            // [n/2 + 1] (sorted position, sector*152 + row) of start hits
+  int32_t *starts;         // [n/2 + 1] sorted positions of the start hits
+  uint32_t *start_bits;    // [n/32 + 1] start hits as a bit mask over the sorted clusters
   int32_t *trk_key;        // [track list capacity] (sector*152 + row) of the track's first cluster
   int32_t *trk_len;        // [track list capacity] chain length
   int32_t *chain;          // [152][track list capacity] sorted positions of each track's clusters
   uint16_t *trk_rl;        // [track list capacity] first row | chain length << 8 (the assignment pass)
   uint32_t *sec_first;     // [nsect] smallest track id of each sector (~0u: none), reset by the row index
   uint32_t *sec_cnt;       // [nsect] tracks of each sector
-  uint64_t *lb_links;      // look-back words, one per 1024-cluster tile
+  uint64_t *lb_links;      // look-back words of the start list and of the hit removal, one per 2048 clusters
   uint64_t *lb_keep;       // look-back words, one per 1024-start tile
   uint32_t *ctr;           // counters (kNCounters)
   uint32_t starts_cap;
@@ -191,15 +193,6 @@ __device__ __forceinline__ uint16_t ld_keep_u16(const uint16_t *addr, uint64_t p
   uint16_t v;
   asm volatile("ld.global.L2::cache_hint.u16 %0, [%1], %2;" : "=h"(v) : "l"(addr), "l"(pol));
   return v;
-}
-__device__ __forceinline__ void st_keep_v4(void *addr, uint4 v, uint64_t pol) {
-  asm volatile("st.global.L2::cache_hint.v4.u32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(addr), "r"(v.x), "r"(v.y),
-               "r"(v.z), "r"(v.w), "l"(pol)
-               : "memory");
-}
-__device__ __forceinline__ void st_keep_v2(void *addr, uint2 v, uint64_t pol) {
-  asm volatile("st.global.L2::cache_hint.v2.u32 [%0], {%1, %2}, %3;" ::"l"(addr), "r"(v.x), "r"(v.y), "l"(pol)
-               : "memory");
 }
 __device__ __forceinline__ void st_keep_u16(uint16_t *addr, uint16_t v, uint64_t pol) {
   asm volatile("st.global.L2::cache_hint.u16 [%0], %1, %2;" ::"l"(addr), "h"(v), "l"(pol) : "memory");

@@ -14,10 +14,17 @@ namespace tpc {
 constexpr int kNbTile = 768;
 constexpr int kNbTileMin = 512;
 inline bool nb_tile_ok(int t) { return t == 512 || t == 768 || t == 1024; }
-// look-back tiles: clusters per tile of the link kernel, start hits per tile of the walk
+// look-back tiles: clusters per tile of the hit removal (the start list takes larger
+// ones), start hits per tile of the walk
 constexpr int kLinkTileN = 2048;
 constexpr int kWalkChains = 1;                  // chains walked together by one thread
 constexpr int kWalkTileN = 256 * kWalkChains;   // start hits per walk tile (256 threads)
+// one buffer holds the start list (n / 2 + 2 positions), then the start mask
+inline size_t start_bits_offset(size_t n) { return ((n / 2 + 2) * 4 + 255) / 256 * 256; }
+inline size_t starts_bytes(size_t n) {
+  const size_t a = (n / 2 + 2) * 8, b = start_bits_offset(n) + (n / 32 + 1) * 4;
+  return a > b ? a : b;
+}
 inline size_t link_tiles(uint32_t n) { return (n + kLinkTileN - 1) / kLinkTileN; }
 inline size_t walk_tiles(uint32_t n) { return (n / 2 + 1 + kWalkTileN - 1) / kWalkTileN; }
 
@@ -32,7 +39,10 @@ void launch_tile_windows(const Args &a, cudaStream_t st);
 // row_cap > 0 lowers the staged window capacity (tests of the global-memory path)
 void launch_neighbours(const Args &a, int row_cap, int sms, cudaStream_t st, bool prune = false);
 void launch_edge_claims(const Args &a, cudaStream_t st);
+// mutual links and start hits, then the list of start hits: one launch for a frame
+// that links_with_list, else two
 void launch_links(const Args &a, int sms, cudaStream_t st);
+bool links_with_list(uint32_t n);
 void launch_walk(const Args &a, int sms, cudaStream_t st);
 // cluster_track, one (sector, row) per CTA step: -1, then each crossing track's id
 void launch_assign(const Args &a, int sms, cudaStream_t st);
