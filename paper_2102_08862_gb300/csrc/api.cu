@@ -700,6 +700,15 @@ extern "C" int tpc_track_timeframe(tpc_tf *tf, const tpc_clusters *cl, const tpc
       if (rc != TPC_OK) return rc;
     }
     TPC_CK(cudaMemsetAsync(tf->f_pred_claim, 0xff, ((size_t)tf->track_list_cap + n) * 4, st));
+    // the start list and mask, the tile table and the claims have been read when the
+    // cross-sector links' index of first clusters takes their place
+    const bool links = tf->cfg.follow == 2 && out->next_track && out->track_capacity > 0;
+    if (links) {
+      a.fl.row_first = tf->tile_off;
+      a.fl.first_time = reinterpret_cast<float *>(a.fl.claim);
+      a.fl.first_own = reinterpret_cast<int32_t *>(a.fl.claim) + n / 2;
+      TPC_CK(cudaMemsetAsync(a.start_bits, 0, ((size_t)n / 32 + 1) * 4, st));
+    }
     launch_follow(a, tf->sms, st);
     stage(tf, st, "follow");
     launch_follow_fit(a, tf->sms, st);
@@ -708,11 +717,12 @@ extern "C" int tpc_track_timeframe(tpc_tf *tf, const tpc_clusters *cl, const tpc
     if (tf->record_ct) TPC_CK(cudaEventRecord(tf->ev_ct, st));  // cluster_track is final
     stage(tf, st, "relabel");
     tf->launches += 9 + !links_with_list(n);  // links, start list, walk, assign, fit, claim reset, time samples, follow, refit, relabel
-    if (tf->cfg.follow == 2 && out->next_track && out->track_capacity > 0) {
+    if (links) {
       TPC_CK(cudaMemsetAsync(tf->f_pred_claim, 0xff, (size_t)tf->track_list_cap * 4, st));
+      TPC_CK(cudaMemsetAsync(a.lb_links, 0, 8 * link_tiles(n), st));
       launch_sector_links(a, tf->sms, st);
       stage(tf, st, "sector_links");
-      tf->launches += 4;  // pred reset, exits, searches, resolve
+      tf->launches += 8;  // mask, pred and look-back resets, list, index, exits, searches, resolve
     }
   }
   TPC_CK(cudaGetLastError());

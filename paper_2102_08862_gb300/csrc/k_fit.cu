@@ -744,6 +744,8 @@ __global__ void __launch_bounds__(256) k_follow_fit(Args a) {
         a.o_row_first[id] = (uint16_t)r0;
         a.o_row_last[id] = (uint16_t)rlast;
         a.o_status[id] = (uint8_t)status;
+        // cross-sector links look for first clusters: this track's, in the mask
+        if (a.fl.row_first) atomicOr(&a.start_bits[start >> 5], 1u << (start & 31));
       }
     }
     __syncthreads();

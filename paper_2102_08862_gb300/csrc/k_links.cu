@@ -111,19 +111,21 @@ __device__ __forceinline__ void stage_links(const Args &a, uint32_t bid, uint32_
   if (bad) raise(a.ctr, kErrRowCap);
 }
 
-// The start hits in cluster order: each thread of a tile takes kListWords words of the
+// The set bits of a mask over the clusters in cluster order (the start hits; the
+// followed tracks' first clusters): each thread of a tile takes kListWords words of the
 // mask (a tile is kListTileN clusters); positions come from a block scan and a
-// decoupled look-back across tiles taken in order from a counter.  The mask is 1/64 of
-// the links' bytes, so the look-back chain is short.
+// decoupled look-back across tiles taken in order from a counter.  The start mask is
+// 1/64 of the links' bytes, so the look-back chain is short.
 constexpr int kListWords = 4;
 constexpr int kListTileN = 32 * kListWords * kThreads;
 static_assert(kListTileN >= kLinkTileN, "look-back words");
-__device__ __forceinline__ void stage_start_list(const Args &a) {
+__device__ __forceinline__ void stage_bit_list(const Args &a, int32_t *__restrict__ out, uint32_t cap,
+                                               int tile_counter, int total_counter) {
   __shared__ uint32_t s_tile, s_prefix;
   __shared__ uint32_t s_warp[kThreads / 32];
   const uint32_t n = a.n, words = (n + 31) / 32, n_tiles = (n + kListTileN - 1) / kListTileN;
   for (;;) {
-    if (threadIdx.x == 0) s_tile = atomicAdd(&a.ctr[kCtrTileLinks], 1u);
+    if (threadIdx.x == 0) s_tile = atomicAdd(&a.ctr[tile_counter], 1u);
     __syncthreads();
     const uint32_t tile = s_tile;
     if (tile >= n_tiles) break;
@@ -143,7 +145,7 @@ __device__ __forceinline__ void stage_start_list(const Args &a) {
       const uint32_t pre = lookback_exclusive(a.lb_links, tile, total, a.ctr, a.spin_limit);
       if (threadIdx.x == 0) {
         s_prefix = pre;
-        if (tile == n_tiles - 1) a.ctr[kCtrStarts] = pre + total;
+        if (tile == n_tiles - 1) a.ctr[total_counter] = pre + total;
       }
     }
     __syncthreads();
@@ -151,9 +153,12 @@ __device__ __forceinline__ void stage_start_list(const Args &a) {
 #pragma unroll
     for (int q = 0; q < kListWords; ++q)
       for (uint32_t b = bits[q]; b; b &= b - 1u, ++pos)
-        if (pos < a.starts_cap) a.starts[pos] = (int32_t)(32u * (w0 + q)) + __ffs((int)b) - 1;
+        if (pos < cap) out[pos] = (int32_t)(32u * (w0 + q)) + __ffs((int)b) - 1;
     __syncthreads();
   }
+}
+__device__ __forceinline__ void stage_start_list(const Args &a) {
+  stage_bit_list(a, a.starts, a.starts_cap, kCtrTileLinks, kCtrStarts);
 }
 
 // A4: one start hit per thread (kWalkChains; walking two or four chains per
@@ -385,6 +390,9 @@ __global__ void __launch_bounds__(kThreads, 8) k_links(Args a, int with_list) {
   stage_start_list(a);
 }
 __global__ void __launch_bounds__(kThreads) k_start_list(Args a) { stage_start_list(a); }
+__global__ void __launch_bounds__(kThreads) k_first_list(Args a) {
+  stage_bit_list(a, a.starts, a.starts_cap, kCtrFirstTile, kCtrFirsts);
+}
 template <bool kSmemRb>
 __global__ void __launch_bounds__(kThreads) k_walk(Args a) {
   stage_walk<kSmemRb>(a, blockIdx.x);
@@ -519,6 +527,11 @@ void launch_links(const Args &a, int sms, cudaStream_t st) {
   if (with_list) return;
   const uint32_t tiles = (a.n + kListTileN - 1) / kListTileN;
   k_start_list<<<tiles < cap ? tiles : cap, kThreads, 0, st>>>(a);
+}
+
+void launch_first_list(const Args &a, int sms, cudaStream_t st) {
+  const uint32_t tiles = (a.n + kListTileN - 1) / kListTileN, cap = (uint32_t)sms * 8u;
+  k_first_list<<<tiles < cap ? (tiles ? tiles : 1u) : cap, kThreads, 0, st>>>(a);
 }
 
 void launch_walk(const Args &a, int sms, cudaStream_t st) {

@@ -83,7 +83,9 @@ enum : int {
   kCtrLinkList = 19,        // cross-sector links: tracks that leave their sector (searched)
   kCtrRegionRows = 20,      // pruned mode: region rows gathered for the dense rescoring
   kCtrLinksDone = 21,       // link kernel: CTAs that have finished
-  kNCounters = 22           // (even: the 8-byte look-back words follow the counters)
+  kCtrFirstTile = 22,       // cross-sector links: next tile of the first clusters' list
+  kCtrFirsts = 23,          // cross-sector links: first clusters listed
+  kNCounters = 24           // (even: the 8-byte look-back words follow the counters)
 };
 
 // A spin-wait gives up after this many polls (with a short sleep between polls,
@@ -162,6 +164,9 @@ struct Args {
     float chi2_link;    // cross-sector links (follow = 2)
     int32_t link_rows;
     int32_t *next;      // [track_capacity] caller's next_track, nullptr when not asked
+    float *first_time;  // cross-sector links: per listed first cluster its time and its track; the clusters
+    int32_t *first_own; // themselves are in `starts`, in cluster order, and `row_first` has each (sector, row)'s
+    int32_t *row_first; // first entry [nkeys + 1]
     int4 *xlist;        // [track_list_cap][2] tracks that leave their sector: (A, exit row, -, -), state at the exit
   } fl;
 };

@@ -43,6 +43,8 @@ void launch_edge_claims(const Args &a, cudaStream_t st);
 // that links_with_list, else two
 void launch_links(const Args &a, int sms, cudaStream_t st);
 bool links_with_list(uint32_t n);
+// the first clusters marked in a.start_bits, in cluster order into a.starts (a.lb_links cleared)
+void launch_first_list(const Args &a, int sms, cudaStream_t st);
 void launch_walk(const Args &a, int sms, cudaStream_t st);
 // cluster_track, one (sector, row) per CTA step: -1, then each crossing track's id
 void launch_assign(const Args &a, int sms, cudaStream_t st);
