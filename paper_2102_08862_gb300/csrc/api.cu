@@ -722,7 +722,7 @@ extern "C" int tpc_track_timeframe(tpc_tf *tf, const tpc_clusters *cl, const tpc
       TPC_CK(cudaMemsetAsync(a.lb_links, 0, 8 * link_tiles(n), st));
       launch_sector_links(a, tf->sms, st);
       stage(tf, st, "sector_links");
-      tf->launches += 8;  // mask, pred and look-back resets, list, index, exits, searches, resolve
+      tf->launches += 10;  // mask, pred and look-back resets, list, index, exit, enter, search, test, resolve
     }
   }
   TPC_CK(cudaGetLastError());

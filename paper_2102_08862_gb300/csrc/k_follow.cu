@@ -55,8 +55,14 @@ struct Fs {
   float c[15];  // covariance, lower triangle
 };
 
+// E of the transport F = I + E has entries (0,2), (0,4), (1,2), (1,3), (1,4), (2,4)
+__host__ __device__ constexpr bool e_at(int i, int k) {
+  return (i == 0 && (k == 2 || k == 4)) || (i == 1 && k >= 2) || (i == 2 && k == 4);
+}
+
 // Transport by dx (either sign); false (state untouched) when |sin phi| would
-// reach 0.999.  F = I + E with E nonzero at (0,2), (0,4), (1,2), (1,3), (1,4), (2,4).
+// reach 0.999.  The products with E's zeros are left out (in floating point the
+// compiler may not: 0 * inf): 55 multiply-adds for the covariance instead of 200.
 __device__ __forceinline__ bool fs_transport(Fs &f, float dx) {
   const float s1 = f.p[2], t = f.p[3];
   const float cv = -kBz * f.p[4];
@@ -68,22 +74,20 @@ __device__ __forceinline__ bool fs_transport(Fs &f, float dx) {
   const float sg = dx < 0.0f ? -1.0f : 1.0f;  // the arc length has the sign of dx
   const float l = sqrtf(dx * dx + dy * dy);
   const float u = 0.5f * cv * l;
-  const float ds = sg * l * asinc(u);
+  float au, ad;
+  asinc_both(u, au, ad);
+  const float ds = sg * l * au;
   const float iD2 = iD * iD;
   const float Fys = dx * (2.0f * D + A * (s1 / c1 + s2 / c2)) * iD2;  // dy/ds1
   const float Fyc = dx * dx * (D + A * s2 / c2) * iD2;                // dy/dc
   const float g = 1.0f / sqrtf((1.0f - u) * (1.0f + u));              // d(arc)/d(chord)
   const float dyl = l > 0.0f ? dy / l : 0.0f;
   float E[5][5];
-#pragma unroll
-  for (int i = 0; i < 5; ++i)
-#pragma unroll
-    for (int j = 0; j < 5; ++j) E[i][j] = 0.0f;
   E[0][2] = Fys;
   E[0][4] = -kBz * Fyc;
   E[1][2] = sg * t * g * dyl * Fys;
   E[1][3] = ds;
-  E[1][4] = -kBz * t * sg * (g * dyl * Fyc + 0.5f * l * l * asinc_d(u));
+  E[1][4] = -kBz * t * sg * (g * dyl * Fyc + 0.5f * l * l * ad);
   E[2][4] = -kBz * dx;
   f.p[0] += dy;
   f.p[1] += t * ds;
@@ -96,7 +100,8 @@ __device__ __forceinline__ bool fs_transport(Fs &f, float dx) {
     for (int j = 0; j < 5; ++j) {
       float acc = f.c[lt(i, j)];
 #pragma unroll
-      for (int k = 0; k < 5; ++k) acc = fmaf(E[i][k], f.c[lt(k, j)], acc);
+      for (int k = 0; k < 5; ++k)
+        if (e_at(i, k)) acc = fmaf(E[i][k], f.c[lt(k, j)], acc);
       FC[i][j] = acc;
     }
 #pragma unroll
@@ -105,7 +110,8 @@ __device__ __forceinline__ bool fs_transport(Fs &f, float dx) {
     for (int j = 0; j <= i; ++j) {
       float acc = FC[i][j];
 #pragma unroll
-      for (int k = 0; k < 5; ++k) acc = fmaf(FC[i][k], E[j][k], acc);
+      for (int k = 0; k < 5; ++k)
+        if (e_at(j, k)) acc = fmaf(FC[i][k], E[j][k], acc);
       f.c[lt(i, j)] = acc;
     }
   return true;
@@ -390,9 +396,10 @@ namespace {
 // the first cluster of a track (with a record) of (sector, row r) under the gate
 // with the smallest (chi2, sorted position); -1 if none.  *owner: its track.  The
 // row's first clusters are a short list of their own in cluster order (k_first_index:
-// 1.3 % of the clusters, 17 per row beyond row 0 on a 5 ms frame), searched by time.
-__device__ int32_t fs_best_first(const Args &a, const Fs &f, int sec, int r, float tref, int32_t *owner) {
-  const int key = sec * kNRows + r;
+// 1.3 % of the clusters, 17 per row beyond row 0 on a 5 ms frame), searched by time;
+// [lo, end) is the row's part of it.
+__device__ __forceinline__ int32_t fs_best_first(const Args &a, const Fs &f, int r, int lo, int end, float tref,
+                                                 int32_t *owner) {
   const float chi2_max = a.fl.chi2_max;
   const float S00 = f.c[0] + kVy, S01 = f.c[1], S11 = f.c[2] + kVz;
   const float half = 0.5f * (float)(row_npads(r) - 1), pitch = (float)row_pitch_um(r) * 1e-4f;
@@ -400,10 +407,6 @@ __device__ int32_t fs_best_first(const Args &a, const Fs &f, int sec, int r, flo
   // the row is searched only where the gate reaches the pad plane (|y| up to
   // npads pitch / 2; chi2 >= r_y^2 / S00)
   if (fabsf(f.p[0]) - 0.5f * (float)row_npads(r) * pitch > sqrtf(chi2_max * S00)) return -1;
-  if (sec >= a.nsect) return -1;
-  const int nf = (int)min(a.ctr[kCtrFirsts], a.starts_cap);
-  int lo = min(max(a.fl.row_first[key], 0), nf);
-  const int end = min(max(a.fl.row_first[key + 1], 0), nf);
   const float idet = 1.0f / (S00 * S11 - S01 * S01);
   const float tp = tref + f.p[1] * (1.0f / kCmPerBin);
   const float w = sqrtf(chi2_max * S11) * (1.0f / kCmPerBin) * 1.001f + 0.01f;
@@ -471,14 +474,13 @@ __device__ __forceinline__ float chi2_5(const float *d, const float *S) {
 
 }  // namespace
 
-// The link search in two kernels, so that the lanes of a warp do the same work:
+// The link search in steps, so that the lanes of a warp do the same work:
 // k_sector_exit gives every followed track one thread that transports its state
 // row by row to the row where it leaves the sector's pad area (most tracks never
 // do, or after a few rows) and lists the tracks that leave it, with that state;
-// k_sector_search gives every listed track one thread for the expensive part
-// (covariance to the exit, rotation, the row-by-row search of the neighbouring
-// sector).  In one kernel a warp's few leaving tracks searched while its other
-// lanes idled (4.6 of 32 lanes active).
+// k_sector_enter takes the listed tracks' covariance there and rotates both into the
+// neighbouring sector's frame; k_sector_search looks for the first cluster of a track
+// row by row; k_sector_test compares the two tracks' states.
 __global__ void __launch_bounds__(kThreads) k_sector_exit(Args a) {
   const uint32_t nf = min(a.ctr[kCtrFollowTracks], a.track_capacity);
   const uint32_t n_up = (nf + 31u) & ~31u;  // whole warps, for the list's shared atomic
@@ -519,19 +521,51 @@ __global__ void __launch_bounds__(kThreads) k_sector_exit(Args a) {
   }
 }
 
-// One thread per listed track: the link proposal to the track continuing it in
-// the neighbouring sector (succ), claimed with atomicMin in pred (reset).
-__global__ void __launch_bounds__(kThreads) k_sector_search(Args a) {
+// The state of a listed track in the neighbouring sector, kept between the kernels of
+// the search in the chain buffer (not read any more, and at least 152 words a track):
+// word k of listed track e is chain[k][e].
+enum : int {
+  kXTrack = 0,   // the track; -1: nothing to search
+  kXSector = 1,  // the neighbouring sector
+  kXRow = 2,     // the next row to search; after the search the row where it ended
+  kXFound = 3,   // after the search: the track found there, -1
+  kXTref = 4,
+  kXAt = 5,      // x of the state (cm)
+  kXState = 6,   // 5 parameters, 15 covariance entries
+  kXWords = 26
+};
+static_assert(kXWords <= kNRows, "words of a track's chain column");
+__device__ __forceinline__ int32_t &x_int(const Args &a, int k, uint32_t e) {
+  return a.chain[(size_t)k * a.track_list_cap + e];
+}
+__device__ __forceinline__ float &x_float(const Args &a, int k, uint32_t e) {
+  return reinterpret_cast<float *>(a.chain)[(size_t)k * a.track_list_cap + e];
+}
+__device__ __forceinline__ void x_store(const Args &a, uint32_t e, const Fs &g) {
+#pragma unroll
+  for (int i = 0; i < 5; ++i) x_float(a, kXState + i, e) = g.p[i];
+#pragma unroll
+  for (int i = 0; i < 15; ++i) x_float(a, kXState + 5 + i, e) = g.c[i];
+}
+__device__ __forceinline__ void x_load(const Args &a, uint32_t e, Fs &g) {
+#pragma unroll
+  for (int i = 0; i < 5; ++i) g.p[i] = x_float(a, kXState + i, e);
+#pragma unroll
+  for (int i = 0; i < 15; ++i) g.c[i] = x_float(a, kXState + 5 + i, e);
+}
+
+// One thread per listed track: its state and covariance at the exit row, rotated into
+// the neighbouring sector's frame.
+__global__ void __launch_bounds__(kThreads) k_sector_enter(Args a) {
   const uint32_t nl = a.ctr[kCtrLinkList];
   const float kCb = 0.93969262f, kSb = 0.34202014f;  // cos, sin of 20 deg
   for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < nl; e += gridDim.x * blockDim.x) {
     const int4 h0 = a.fl.xlist[2 * (size_t)e], h1 = a.fl.xlist[2 * (size_t)e + 1];
     const uint32_t A = (uint32_t)h0.x;
     int exit_row = h0.y;
-    int32_t prop = -1;
+    bool enters = false;
     const int rl = a.o_row_last[A];
     const int sec = a.o_sector[A];
-    const float tref = a.t_ref[A];
     Fs f;
     fs_load_record(a, A, f);
     // the covariance is transported from the record to the exit in one step (the
@@ -592,36 +626,120 @@ __global__ void __launch_bounds__(kThreads) k_sector_search(Args a) {
             g.c[lt(i, j)] = acc;
           }
         const int side = sec / 18, ls = sec % 18;
-        const int s2ec = side * 18 + (up ? (ls + 1) % 18 : (ls + 17) % 18);
         int r0 = 0;
         while (r0 < kNRows && row_x(r0) < xr) ++r0;
-        float xcur = xr;
-        for (int r = r0; r < kNRows && r < r0 + a.fl.link_rows; ++r) {
-          if (!fs_transport(g, row_x(r) - xcur)) break;
-          xcur = row_x(r);
-          int32_t B;
-          const int32_t c = fs_best_first(a, g, s2ec, r, tref, &B);
-          if (c < 0) continue;
-          if (a.o_status[B] == 0) {
-            Fs h;
-            fs_load_record(a, B, h);
-            if (fs_transport(h, row_x(r) - a.x[B])) {
-              h.p[1] += kCmPerBin * (a.t_ref[B] - tref);
-              float d[5], S[15];
-#pragma unroll
-              for (int i = 0; i < 5; ++i) d[i] = g.p[i] - h.p[i];
-#pragma unroll
-              for (int i = 0; i < 15; ++i) S[i] = g.c[i] + h.c[i];
-              const float q5 = chi2_5(d, S);
-              if (q5 >= 0.0f && q5 <= a.fl.chi2_link) prop = B;
-            }
-          }
-          break;
-        }
+        enters = r0 < kNRows;
+        x_int(a, kXSector, e) = side * 18 + (up ? (ls + 1) % 18 : (ls + 17) % 18);
+        x_int(a, kXRow, e) = r0;
+        x_float(a, kXTref, e) = a.t_ref[A];
+        x_float(a, kXAt, e) = xr;
+        x_store(a, e, g);
       }
     }
-    a.fl.succ[A] = prop;
-    if (prop >= 0) atomicMin(&a.fl.pred[prop], A);
+    x_int(a, kXTrack, e) = enters ? (int32_t)A : -1;
+    x_int(a, kXFound, e) = -1;
+    a.fl.succ[A] = -1;
+  }
+}
+
+// The row-by-row search: a lane searches one track at a time, one row per pass of its
+// warp's loop, and takes the next one from a counter when enough lanes of the warp are
+// done (the wait for the new states is the warp's), because the searches differ in
+// length by up to 150 rows.  Search of a 5 ms frame (0.2 M tracks): one thread per
+// track 0.39 ms with 6 of 32 lanes active; so, and with the transport's zero products
+// left out, 0.25 with 11 (rows with and without first clusters in reach diverge).  2
+// CTAs per SM take 0.07 ms more, 8 take 0.05.
+constexpr int kSearchThreads = 128;
+constexpr int kSearchCtasPerSm = 6;
+constexpr int kSearchRefill = 4;  // idle lanes that make a warp take new tracks
+__global__ void __launch_bounds__(kSearchThreads) k_sector_search(Args a) {
+  const uint32_t nl = a.ctr[kCtrLinkList];
+  const int lane = threadIdx.x & 31;
+  bool active = false, more = true;
+  uint32_t e = 0;
+  int r = 0, rend = 0;
+  float tref = 0.0f, xcur = 0.0f;
+  Fs g;
+  // the list's parts of rows r and r + 1 are [b0, b1) and [b1, b2): a pass loads what
+  // the row after next needs and touches the next row's first probe, so that its
+  // search finds both there (a long search's passes follow one another: their
+  // latency is the kernel's)
+  const int nf = (int)min(a.ctr[kCtrFirsts], a.starts_cap);
+  const int32_t *bound = a.fl.row_first;
+  int b0 = 0, b1 = 0, b2 = 0, key = 0;
+  auto row_bound = [&](int k) { return min(max(bound[min(k, a.nkeys)], 0), nf); };
+  for (;;) {
+    const unsigned idle = __ballot_sync(0xffffffffu, !active);
+    if (more && __popc(idle) >= kSearchRefill) {
+      uint32_t base = 0;
+      if (lane == 0) base = atomicAdd(&a.ctr[kCtrLinkNext], (uint32_t)__popc(idle));
+      base = __shfl_sync(0xffffffffu, base, 0);
+      more = base + (uint32_t)__popc(idle) < nl;
+      if (!active) {
+        e = base + (uint32_t)__popc(idle & ((1u << lane) - 1u));
+        if (e < nl && x_int(a, kXTrack, e) >= 0) {
+          const int sec = x_int(a, kXSector, e);
+          active = sec < a.nsect;
+          r = x_int(a, kXRow, e);
+          key = sec * kNRows + r;
+          b0 = row_bound(key);
+          b1 = row_bound(key + 1);
+          b2 = row_bound(key + 2);
+          rend = min(kNRows, r + a.fl.link_rows);
+          tref = x_float(a, kXTref, e);
+          xcur = x_float(a, kXAt, e);
+          x_load(a, e, g);
+        }
+      }
+      continue;
+    }
+    if (idle == 0xffffffffu) break;  // (and no more tracks)
+    if (!active) continue;
+    const int b3 = row_bound(key + 3);
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(a.fl.first_time + ((b1 + b2) >> 1)));
+    active = r < rend && fs_transport(g, row_x(r) - xcur);
+    if (active) {
+      xcur = row_x(r);
+      int32_t B;
+      if (fs_best_first(a, g, r, b0, b1, tref, &B) >= 0) {
+        x_int(a, kXRow, e) = r;
+        x_int(a, kXFound, e) = B;
+        x_store(a, e, g);
+        active = false;
+      }
+      ++r;
+      ++key;
+      b0 = b1;
+      b1 = b2;
+      b2 = b3;
+    }
+  }
+}
+
+// One thread per listed track: the link test with the track found, and the proposal to
+// it (succ), claimed with atomicMin in pred (reset).
+__global__ void __launch_bounds__(kThreads) k_sector_test(Args a) {
+  const uint32_t nl = a.ctr[kCtrLinkList];
+  for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < nl; e += gridDim.x * blockDim.x) {
+    const int32_t A = x_int(a, kXTrack, e), B = x_int(a, kXFound, e);
+    if (A < 0 || B < 0 || a.o_status[B] != 0) continue;
+    const int r = x_int(a, kXRow, e);
+    const float tref = x_float(a, kXTref, e);
+    Fs g, h;
+    x_load(a, e, g);
+    fs_load_record(a, (uint32_t)B, h);
+    if (!fs_transport(h, row_x(r) - a.x[B])) continue;
+    h.p[1] += kCmPerBin * (a.t_ref[B] - tref);
+    float d[5], S[15];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) d[i] = g.p[i] - h.p[i];
+#pragma unroll
+    for (int i = 0; i < 15; ++i) S[i] = g.c[i] + h.c[i];
+    const float q5 = chi2_5(d, S);
+    if (q5 >= 0.0f && q5 <= a.fl.chi2_link) {
+      a.fl.succ[A] = B;
+      atomicMin(&a.fl.pred[B], (uint32_t)A);
+    }
   }
 }
 
@@ -658,7 +776,9 @@ void launch_sector_links(const Args &a, int sms, cudaStream_t st) {
   launch_first_list(a, sms, st);
   k_first_index<<<sms * 4, kThreads, 0, st>>>(a);
   k_sector_exit<<<sms * 4, kThreads, 0, st>>>(a);
-  k_sector_search<<<sms * 4, kThreads, 0, st>>>(a);
+  k_sector_enter<<<sms * 4, kThreads, 0, st>>>(a);
+  k_sector_search<<<sms * kSearchCtasPerSm, kSearchThreads, 0, st>>>(a);
+  k_sector_test<<<sms * 4, kThreads, 0, st>>>(a);
   k_sector_links_resolve<<<sms * 4, kThreads, 0, st>>>(a);
 }
 

@@ -21,5 +21,17 @@ __device__ __forceinline__ float asinc_d(float u) {
   if (fabsf(u) < 0.05f) return u * (1.0f / 3.0f + u2 * (0.3f + u2 * (15.0f / 56.0f + u2 * (35.0f / 144.0f))));
   return (u / sqrtf((1.0f - u) * (1.0f + u)) - asinf(u)) / u2;
 }
+// both of them, with one branch and one asinf
+__device__ __forceinline__ void asinc_both(float u, float &f, float &d) {
+  const float u2 = u * u;
+  if (fabsf(u) < 0.05f) {
+    f = 1.0f + u2 * (1.0f / 6.0f + u2 * (3.0f / 40.0f + u2 * (5.0f / 112.0f)));
+    d = u * (1.0f / 3.0f + u2 * (0.3f + u2 * (15.0f / 56.0f + u2 * (35.0f / 144.0f))));
+  } else {
+    const float as = asinf(u);
+    f = as / u;
+    d = (u / sqrtf((1.0f - u) * (1.0f + u)) - as) / u2;
+  }
+}
 
 }  // namespace tpc

@@ -85,7 +85,8 @@ enum : int {
   kCtrLinksDone = 21,       // link kernel: CTAs that have finished
   kCtrFirstTile = 22,       // cross-sector links: next tile of the first clusters' list
   kCtrFirsts = 23,          // cross-sector links: first clusters listed
-  kNCounters = 24           // (even: the 8-byte look-back words follow the counters)
+  kCtrLinkNext = 24,        // cross-sector links: next listed track to search
+  kNCounters = 26           // (even: the 8-byte look-back words follow the counters)
 };
 
 // A spin-wait gives up after this many polls (with a short sleep between polls,
