@@ -43,6 +43,9 @@ constexpr int kMaxRanges = 8;             // sector ranges of a pipelined host-b
 constexpr uint32_t kRangeMinClusters = 1u << 22;  // smaller frames are copied in one piece
 constexpr int kRanges = 3;  // measured on the 10 ms frame: 3 ranges 7.45e9 clusters/s end to end, 4: 7.30e9, 6: 6.66e9, 8: 6.15e9
 
+constexpr int kPinnedCounters = 32;  // (of the 64 words of the handle's page-locked buffer)
+static_assert(kPinnedCounters + kNCounters <= 64, "page-locked words");
+
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 }  // namespace
@@ -82,7 +85,8 @@ struct tpc_tf {
   uint8_t *h_status = nullptr;
   int32_t *h_next = nullptr;  // follow = 2 only
   uint32_t *h_ntracks = nullptr;
-  uint32_t *pinned = nullptr;  // [0] n_tracks, [1] error word, [4 + k] / [16 + k] a range's error word / running track count
+  uint32_t *pinned = nullptr;  // [0] n_tracks, [1] error word, [4 + k] / [16 + k] a range's error word / running track
+                               // count, [kPinnedCounters ...] a call's counters
   cudaEvent_t ev[kMaxStages + 1];
   const char *ev_name[kMaxStages];
   int n_ev = 0;
@@ -120,8 +124,8 @@ struct tpc_tf {
   // host-buffer calls: cluster_track is copied back on aux_stream as soon as it is
   // final (after the assignment pass; after relabelling in follow mode), while the fit runs
   cudaStream_t aux_stream = nullptr;
-  // the cluster_track assignment runs on side_stream while the fit runs on the
-  // call's stream (both only read the chains); forked and joined by events
+  // host-buffer calls: the cluster_track assignment runs on side_stream while the fit
+  // runs on the call's stream (both only read the chains); forked and joined by events
   cudaStream_t side_stream = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   cudaEvent_t ev_ct = nullptr;
@@ -212,7 +216,7 @@ static std::vector<Part> plan_arena(tpc_tf *tf, const tpc_tf_config *cfg) {
   const size_t N = tf->N;
   const bool fol = cfg->follow != 0;
   const size_t TL = tf->track_list_cap;
-  tf->reset_bytes_max = kNCounters * 4 + 8 * (link_tiles(tf->N) + walk_tiles(tf->N) + 2 +
+  tf->reset_bytes_max = reset_words(tf->nkeys) * 4 + 8 * (link_tiles(tf->N) + walk_tiles(tf->N) + 2 +
                                               (fol ? follow_tiles(tf->N, cfg->n_min, tf->track_list_cap) : 0));
   std::vector<Part> parts = {
       {(void **)&tf->row_begin, (size_t)(tf->nkeys + 1) * 4},
@@ -451,7 +455,8 @@ static void fill_args(tpc_tf *tf, uint32_t n, const tpc_tracks *out, Args &a) {
   a.chain = tf->chain;
   a.ctr = tf->reset;
   const size_t tiles_l = link_tiles(n);
-  a.lb_links = reinterpret_cast<uint64_t *>(reinterpret_cast<char *>(tf->reset) + kNCounters * 4);
+  a.key_first = tf->reset + kNCounters;
+  a.lb_links = reinterpret_cast<uint64_t *>(tf->reset + reset_words(tf->nkeys));
   a.lb_keep = a.lb_links + tiles_l;
   a.starts_cap = n / 2 + 1;
   a.track_list_cap = tf->track_list_cap;
@@ -524,7 +529,7 @@ static int enqueue_linking(tpc_tf *tf, const tpc_clusters *cl, Args &a, cudaStre
   if (tf->cfg.profile_stages) cudaEventRecord(tf->ev[0], st);
   TPC_CK(cudaMemsetAsync(
       tf->reset, 0,
-      kNCounters * 4 +
+      reset_words(tf->nkeys) * 4 +
           8 * (link_tiles(n) + walk_tiles(n) + (tf->cfg.follow ? follow_tiles(n, tf->cfg.n_min, tf->track_list_cap) : 0)),
       st));
   ++tf->launches;
@@ -548,12 +553,11 @@ static int enqueue_linking(tpc_tf *tf, const tpc_clusters *cl, Args &a, cudaStre
     stage(tf, st, "sort");
   }
   launch_quantize(a, tf->sms, st);
-  launch_row_index(a, st);
   launch_tile_windows(a, st);
   stage(tf, st, "ingest");
   launch_neighbours(a, tf->cfg.row_cap, tf->sms, st, prune);
   stage(tf, st, "neighbours");
-  tf->launches += 4;
+  tf->launches += 3;
   if (prune) {
     launch_region_rescore(a, tf->mlp, tf->mlp_head, tf->rr_feat, tf->rr_meta, tf->rr_cost, tf->rr_logit,
                           tf->logit_tau, tf->sms, tf->cfg.mlp_engine, st);
@@ -578,7 +582,7 @@ static int enqueue_persistent(tpc_tf *tf, const tpc_clusters *cl, Args &a, cudaS
   tf->n_ev = 0;
   tf->launches = 0;
   if (tf->cfg.profile_stages) cudaEventRecord(tf->ev[0], st);
-  TPC_CK(cudaMemsetAsync(tf->reset, 0, kNCounters * 4 + 8 * (link_tiles(n) + walk_tiles(n)), st));
+  TPC_CK(cudaMemsetAsync(tf->reset, 0, reset_words(tf->nkeys) * 4 + 8 * (link_tiles(n) + walk_tiles(n)), st));
   ++tf->launches;
   if (sorted) {
     a.sector = cl->sector;
@@ -607,12 +611,12 @@ static int enqueue_persistent(tpc_tf *tf, const tpc_clusters *cl, Args &a, cudaS
   return TPC_OK;
 }
 
-// A4 assignment and A5 fit.  Both only read the chains, so the assignment runs on
-// the side stream while the fit runs on st (with stage profiling they run one
-// after the other on st, so that each has its own time).  cluster_track is final
-// when the assignment ends (ev_ct, for the host-buffer path).
+// A4 assignment and A5 fit, which both only read the chains: one launch for the two
+// (with stage profiling, or a warp per track, they run one after the other).  For the
+// host-buffer path cluster_track has to be final early (ev_ct: it is copied back while
+// the fit runs), so there the assignment runs on the side stream beside the fit.
 static int enqueue_assign_fit(tpc_tf *tf, const Args &a, cudaStream_t st) {
-  if (tf->cfg.profile_stages) {
+  if (tf->cfg.profile_stages || (tf->cfg.fit_variant == TPC_FIT_WARP && !tf->record_ct)) {
     launch_assign(a, tf->sms, st);
     if (tf->record_ct) TPC_CK(cudaEventRecord(tf->ev_ct, st));
     stage(tf, st, "assign");
@@ -620,10 +624,15 @@ static int enqueue_assign_fit(tpc_tf *tf, const Args &a, cudaStream_t st) {
     stage(tf, st, "fit");
     return TPC_OK;
   }
+  if (!tf->record_ct) {
+    launch_fit_assign(a, tf->sms, st);
+    --tf->launches;  // (counted as two)
+    return TPC_OK;
+  }
   TPC_CK(cudaEventRecord(tf->ev_fork, st));
   TPC_CK(cudaStreamWaitEvent(tf->side_stream, tf->ev_fork, 0));
   launch_assign(a, tf->sms, tf->side_stream);
-  if (tf->record_ct) TPC_CK(cudaEventRecord(tf->ev_ct, tf->side_stream));
+  TPC_CK(cudaEventRecord(tf->ev_ct, tf->side_stream));
   TPC_CK(cudaEventRecord(tf->ev_join, tf->side_stream));
   launch_fit(a, tf->sms, tf->cfg.fit_variant, st);
   TPC_CK(cudaStreamWaitEvent(st, tf->ev_join, 0));
@@ -728,12 +737,11 @@ extern "C" int tpc_track_timeframe(tpc_tf *tf, const tpc_clusters *cl, const tpc
   TPC_CK(cudaGetLastError());
   tf->last_args = a;
   if (out->n_tracks_host) {
-    TPC_CK(cudaMemcpyAsync(tf->pinned, tf->reset + (tf->cfg.follow ? kCtrFollowTracks : kCtrTracks), 4,
-                           cudaMemcpyDeviceToHost, st));
-    TPC_CK(cudaMemcpyAsync(tf->pinned + 1, tf->reset + kCtrErr, 4, cudaMemcpyDeviceToHost, st));
+    uint32_t *ctr = tf->pinned + kPinnedCounters;  // the counters in one copy: the count and the error word
+    TPC_CK(cudaMemcpyAsync(ctr, tf->reset, kNCounters * 4, cudaMemcpyDeviceToHost, st));
     TPC_CK(cudaStreamSynchronize(st));
-    *out->n_tracks_host = tf->pinned[0];
-    return map_err(tf->pinned[1]);
+    *out->n_tracks_host = ctr[tf->cfg.follow ? kCtrFollowTracks : kCtrTracks];
+    return map_err(ctr[kCtrErr]);
   }
   return TPC_OK;
 }

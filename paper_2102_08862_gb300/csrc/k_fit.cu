@@ -31,6 +31,7 @@
 // This file is compiled with approximate FP32 division and square root (a few
 // ulp): the filter's error stays far inside the 1e-4 tolerance, and the stage
 // runs 16 % faster than with IEEE-rounded division.
+#include "assign_dev.cuh"
 #include "kf_dev.cuh"
 #include "tpc_dev.cuh"
 #include "tpc_internal.h"
@@ -292,17 +293,18 @@ __device__ __forceinline__ void kf_covariance(const Kf &k, float *c) {
 // shared memory (bitonic), so that the lanes of a warp fit chains of similar
 // length and finish together; the chain reads of a step stay inside the block's
 // 256 columns (1 KB, cached in L1).
+template <int THREADS>
 __device__ __forceinline__ void stage_fit(const Args &a, uint32_t bid, uint32_t nblk) {
-  __shared__ uint32_t s_key[256];
+  __shared__ uint32_t s_key[THREADS];
   const uint32_t nt = min(min(a.ctr[kCtrTracks], a.track_list_cap), a.track_capacity);
   const size_t stride = a.track_list_cap;
-  for (uint32_t t0 = bid * 256; t0 < nt; t0 += nblk * 256) {
+  for (uint32_t t0 = bid * THREADS; t0 < nt; t0 += nblk * THREADS) {
     {
       const uint32_t tt = t0 + threadIdx.x;
       const uint32_t len = tt < nt ? (uint32_t)a.trk_len[tt] : 0u;
       s_key[threadIdx.x] = (len << 8) | threadIdx.x;
       __syncthreads();
-      for (int k = 2; k <= 256; k <<= 1)
+      for (int k = 2; k <= THREADS; k <<= 1)
         for (int j = k >> 1; j > 0; j >>= 1) {
           const int i = threadIdx.x, ixj = i ^ j;
           if (ixj > i) {
@@ -390,9 +392,30 @@ __device__ __forceinline__ void stage_fit(const Args &a, uint32_t bid, uint32_t 
 // than k_fit_thread (one filter per warp instead of per lane), which the
 // coalesced chain loads do not pay back: the thread kernel stays the default.
 #ifndef TPC_STAGES_ONLY
-__global__ void __launch_bounds__(256) k_fit_thread(Args a) { stage_fit(a, blockIdx.x, gridDim.x); }
+constexpr int kFitThreads = 256;
+__global__ void __launch_bounds__(kFitThreads) k_fit_thread(Args a) { stage_fit<kFitThreads>(a, blockIdx.x, gridDim.x); }
+
+// The fit, then the cluster_track assignment, which reads the same chains: one launch
+// whose first fit_blocks blocks fit and whose others assign.  The fit is the longer
+// chain and its blocks few on small frames, so they come first and land on one SM each;
+// run on two streams, the assignment's blocks took the SMs first whenever its launch
+// arrived first, and the fit's shared what was left.  A call, two streams -> one launch:
+// one sector of a 10 ms frame 0.282 -> 0.248 ms, 2 ms frame 0.436 -> 0.400, 10 ms pruned
+// 1.617 -> 1.559.  (Neither this launch nor the walk overlaps its predecessor: a few
+// heavy blocks placed where the predecessor's end would bunch on few SMs, which took a
+// 2 ms frame to 0.57 ms.)
+// clusters of a row built in shared memory at once: 26 KB holds a row of a 10 ms frame
+// and leaves the fit its L1 cache (10 ms frame, a call: 16 KB 1632 us, 26 KB 1559, 32 KB
+// 1574, 48 KB 2149)
+constexpr int kFitAssignCap = 6656;
+__global__ void __launch_bounds__(kFitThreads) k_fit_assign(Args a, uint32_t fit_blocks) {
+  extern __shared__ int32_t assign_buf[];
+  if (blockIdx.x < fit_blocks) stage_fit<kFitThreads>(a, blockIdx.x, fit_blocks);
+  else stage_assign<kFitAssignCap>(a, blockIdx.x - fit_blocks, gridDim.x - fit_blocks, assign_buf);
+}
 
 __global__ void __launch_bounds__(256) k_fit_warp(Args a) {
+  pdl_begin();
   const uint32_t nt = min(min(a.ctr[kCtrTracks], a.track_list_cap), a.track_capacity);
   const size_t stride = a.track_list_cap;
   const int lane = threadIdx.x & 31;
@@ -479,14 +502,30 @@ __global__ void __launch_bounds__(256) k_fit_warp(Args a) {
 }
 
 void launch_fit(const Args &a, int sms, int variant, cudaStream_t st) {
-  if (variant == TPC_FIT_WARP) k_fit_warp<<<sms * 8, 256, 0, st>>>(a);
-  else {
+  if (variant == TPC_FIT_WARP) {
+    launch_pdl(k_fit_warp, (uint32_t)sms * 8u, 256, 0, st, a.n, a);
+  } else {
     // one block per 256-track group of the list (blocks past the track count exit at
     // once; the grid-stride loop covers lists of more than 65535 groups), so that
     // the hardware hands groups to SMs as they free up
-    const size_t groups = ((size_t)a.track_list_cap + 255) / 256;
-    k_fit_thread<<<(unsigned)(groups < 65535 ? (groups ? groups : 1) : 65535), 256, 0, st>>>(a);
+    const size_t groups = ((size_t)a.track_list_cap + kFitThreads - 1) / kFitThreads;
+    k_fit_thread<<<(unsigned)(groups < 65535 ? (groups ? groups : 1) : 65535), kFitThreads, 0, st>>>(a);
   }
+}
+
+void launch_fit_assign(const Args &a, int sms, cudaStream_t st) {
+  // a block per 256-track group, as above, up to one track in 48 clusters (they average
+  // 70); denser frames take groups in turn.  Empty blocks would only delay the assignment.
+  const size_t groups = ((size_t)a.track_list_cap + kFitThreads - 1) / kFitThreads;
+  const size_t usual = (size_t)a.n / (48 * kFitThreads) + 1;
+  const uint32_t fit = (uint32_t)(groups < usual ? (groups ? groups : 1) : usual);
+  k_fit_assign<<<fit + assign_blocks(a, sms), kFitThreads, kFitAssignCap * 4, st>>>(a, fit);
+}
+
+int fit_assign_prepare() {
+  return cudaFuncSetAttribute(k_fit_assign, cudaFuncAttributeMaxDynamicSharedMemorySize, kFitAssignCap * 4) == cudaSuccess
+             ? 0
+             : -1;
 }
 
 // ------------------------------------------------------- followed tracks

@@ -1,141 +1,93 @@
-// k_index.cu -- A0 ingest for input sorted by (sector, row, time, pad): the
-// (sector, row) index row_begin[] and the largest row, which selects the
-// neighbour kernel (staged rows in shared memory, or global memory).
+// k_index.cu -- A0 ingest of the sorted clusters in one pass: validation,
+// quantisation and the (sector, row) index row_begin[] with the neighbour kernel's
+// tile table.
 //
 // The paper processes a whole ~10 ms time frame at once, held in GPU memory
-// (Sec. 1); clusters arrive sorted by row and time from the clusteriser, so the
-// index is a lower-bound search per (sector, row) key instead of a pass over
-// every cluster.  Full validation of every cluster happens in the neighbour
-// kernels, which read every cluster anyway.
+// (Sec. 1); clusters arrive sorted by row and time from the clusteriser, so every
+// (sector, row) begins where the key of a cluster differs from its predecessor's, which
+// the validation compares anyway: the pass records those clusters, and its last CTA
+// turns them into the tables.
 #include "tpc_dev.cuh"
 #include "tpc_internal.h"
 
 namespace tpc {
 
-// first i in [0, n) with key(i) >= k, key = sector * 152 + row; one warp, 32-ary
-// search (five rounds of 32 parallel probes for 32M clusters).  With unsorted
-// keys the result is still inside [0, n].
-__device__ __forceinline__ uint32_t warp_lower_bound_key(const uint16_t *sector, const uint16_t *row, uint32_t n,
-                                                         int k) {
-  const int lane = threadIdx.x & 31;
-  uint32_t lo = 0, hi = n;
-  while (hi - lo > 32) {
-    const uint32_t step = (hi - lo + 31) / 32;
-    const uint32_t p = lo + (uint32_t)lane * step;
-    bool less = false;
-    if (p < hi) less = (int)sector[p] * kNRows + (int)row[p] < k;
-    const unsigned b = __ballot_sync(0xffffffffu, less);
-    const int c = __popc(b);
-    const uint32_t nlo = c > 0 ? lo + (uint32_t)(c - 1) * step + 1 : lo;
-    uint32_t nhi = lo + (uint32_t)c * step;
-    if (c == 32 || nhi > hi) nhi = hi;
-    lo = nlo;
-    hi = nhi < nlo ? nlo : nhi;
-  }
-  bool less = false;
-  const uint32_t p = lo + (uint32_t)lane;
-  if (p < hi) less = (int)sector[p] * kNRows + (int)row[p] < k;
-  return lo + (uint32_t)__popc(__ballot_sync(0xffffffffu, less));
-}
-
-// The row index in two parts, so that the persistent kernel can run them with a
-// grid barrier between: (1) one warp per (sector, row) key, warps taken in turn
-// by blocks bid, bid + nblk, ...; (2) one block: the largest row, the
-// monotonicity check and the first neighbour tile of every row (each thread owns
-// a contiguous block of keys; block-wide exclusive scan).
-__device__ __forceinline__ void stage_row_index_keys(const Args &a, uint32_t bid, uint32_t nblk) {
-  const int lane = threadIdx.x & 31;
-  const int wpb = (int)(blockDim.x >> 5);
-  for (int warp = (int)bid * wpb + (int)(threadIdx.x >> 5); warp <= a.nkeys; warp += (int)nblk * wpb) {
-    const uint32_t r = warp_lower_bound_key(a.sector, a.row, a.n, warp);
-    if (lane == 0) {
-      a.row_begin[warp] = (int32_t)r;
-      // clusters with a key >= nsect*152 sit after row_begin[nkeys]: invalid input
-      if (warp == a.nkeys && r != a.n) raise(a.ctr, kErrInput);
-    }
-  }
-}
-
+// One block: row_begin from the recorded first clusters (key_first: index + 1, 0 for a
+// key without clusters; a key begins where the next one present does), the largest row
+// and the first neighbour tile of every row.  Each thread owns a contiguous block of
+// keys, read at L2 (ld.cg: other blocks wrote them) kBatch at a time, so that one round
+// trip serves a whole frame's 22 keys per thread; block-wide scans join the blocks.
+// With unsorted input (an error) the minima keep row_begin monotone and inside [0, n].
 __device__ __forceinline__ void stage_row_index_table(const Args &a) {
+  constexpr int kBatch = 24;
+  __shared__ int32_t s_min[256];
+  __shared__ uint32_t s_warp[8];
   __shared__ int s_max[8];
-  __shared__ int s_scan[256];
-  const int lane = threadIdx.x & 31;
-  for (int q = threadIdx.x; q < a.nsect; q += blockDim.x) {  // the walk's per-sector track ranges
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  for (int q = tid; q < a.nsect; q += 256) {  // the walk's per-sector track ranges
     a.sec_first[q] = ~0u;
     a.sec_cnt[q] = 0u;
   }
-  // row_begin was written by the other blocks of this launch: read at L2 (ld.cg),
-  // eight keys' entries per round trip
-  const int32_t *rbg = a.row_begin;
   const int nkeys = a.nkeys, tile = a.nb_tile;
-  const int per = (nkeys + blockDim.x - 1) / blockDim.x;
-  const int k0 = threadIdx.x * per, k1 = min(nkeys, k0 + per);
+  const int per = (nkeys + 255) / 256, k0 = min(nkeys, tid * per), k1 = min(nkeys, k0 + per);
+  const int32_t n = (int32_t)a.n;
+  // first present cluster of this thread's keys, then of all keys behind them
+  int32_t mine = n;
+  for (int k = k0; k < k1; k += kBatch) {
+    uint32_t v[kBatch];
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) v[u] = k + u < k1 ? __ldcg(a.key_first + k + u) : 0u;
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u)
+      if (v[u]) mine = min(mine, (int32_t)v[u] - 1);
+  }
+  int32_t x = mine;
+  for (int o = 1; o < 32; o <<= 1) x = min(x, __shfl_down_sync(0xffffffffu, x, o));  // (past lane 31: its own value)
+  if (lane == 0) s_min[w] = x;
+  __syncthreads();
+  int32_t next = __shfl_down_sync(0xffffffffu, x, 1);
+  if (lane == 31) next = n;
+  for (int q = w + 1; q < 8; ++q) next = min(next, s_min[q]);
+  // row_begin of this thread's keys, from the last one back, and its tiles
   int mx = 0, ntile = 0;
-  for (int k = k0; k < k1; k += 8) {
-    int32_t v[9];
+  int32_t run = next;
+  for (int ke = k1; ke > k0; ke -= kBatch) {
+    uint32_t v[kBatch];
 #pragma unroll
-    for (int u = 0; u < 9; ++u) v[u] = k + u <= k1 ? __ldcg(rbg + k + u) : 0;
+    for (int u = 0; u < kBatch; ++u) v[u] = ke - 1 - u >= k0 ? __ldcg(a.key_first + ke - 1 - u) : 0u;
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (k + u < k1) {
-        if (v[u + 1] < v[u]) raise(a.ctr, kErrInput);
-        const int c = max(0, v[u + 1] - v[u]);
+    for (int u = 0; u < kBatch; ++u)
+      if (ke - 1 - u >= k0) {
+        const int32_t begin = v[u] ? min(run, (int32_t)v[u] - 1) : run;
+        const int c = run - begin;
+        a.row_begin[ke - 1 - u] = begin;
         mx = max(mx, c);
         ntile += (c + tile - 1) / tile;
+        run = begin;
       }
   }
-  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if (lane == 0) s_max[threadIdx.x >> 5] = mx;
-  s_scan[threadIdx.x] = ntile;
-  __syncthreads();
-  for (int o = 1; o < (int)blockDim.x; o <<= 1) {
-    const int v = threadIdx.x >= (unsigned)o ? s_scan[threadIdx.x - o] : 0;
-    __syncthreads();
-    s_scan[threadIdx.x] += v;
-    __syncthreads();
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (lane == 0) s_max[w] = mx;
+  uint32_t total;
+  uint32_t off = block_exclusive_scan<256>((uint32_t)ntile, s_warp, &total);
+  int32_t b = run;  // row_begin[k0] (written above by this thread, as are its other keys)
+  for (int k = k0; k < k1; ++k) {
+    const int32_t e = k + 1 < k1 ? a.row_begin[k + 1] : next;
+    a.tile_off[k] = (int32_t)off;
+    off += (uint32_t)((e - b + tile - 1) / tile);
+    b = e;
   }
-  int off = s_scan[threadIdx.x] - ntile;
-  for (int k = k0; k < k1; k += 8) {
-    int32_t v[9];
-#pragma unroll
-    for (int u = 0; u < 9; ++u) v[u] = k + u <= k1 ? __ldcg(rbg + k + u) : 0;
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (k + u < k1) {
-        a.tile_off[k + u] = off;
-        off += (max(0, v[u + 1] - v[u]) + tile - 1) / tile;
-      }
-  }
-  if (threadIdx.x == blockDim.x - 1) {
-    a.tile_off[nkeys] = s_scan[threadIdx.x];
-    a.ctr[kCtrTiles] = (uint32_t)s_scan[threadIdx.x];
-    if ((uint32_t)s_scan[threadIdx.x] > a.tile_cap) raise(a.ctr, kErrInternal);
-  }
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
+    a.row_begin[nkeys] = n;
+    a.tile_off[nkeys] = (int32_t)total;
+    a.ctr[kCtrTiles] = total;
+    if (total > a.tile_cap) raise(a.ctr, kErrInternal);
     int m = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = max(m, s_max[w]);
+    for (int q = 0; q < 8; ++q) m = max(m, s_max[q]);
     a.ctr[kCtrMaxRow] = (uint32_t)m;
     if (m > 65534) raise(a.ctr, kErrRowCap);  // row-local links are 16-bit
   }
 }
-
-#ifndef TPC_STAGES_ONLY
-// one launch: every key has its warp; the last block to finish builds the table
-__global__ void __launch_bounds__(256) k_row_index(Args a) {
-  stage_row_index_keys(a, blockIdx.x, gridDim.x);
-  __shared__ bool s_last;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned d = atomicAdd(&a.ctr[kCtrIndexDone], 1u);
-    s_last = (d == gridDim.x - 1);
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  stage_row_index_table(a);
-}
-#endif
 
 // A0 validation and quantisation, one pass over the sorted clusters: every
 // cluster must have sector < nsect, row < 152, a pad and a time inside the
@@ -153,8 +105,9 @@ struct QCheck {
   int kp;
   float tp, pp;
   bool bad;
-  __device__ __forceinline__ void step(int key, float t, float p, bool first_of_array) {
-    if (!first_of_array && !(kp < key || (kp == key && (tp < t || (tp == t && pp <= p))))) bad = true;
+  __device__ __forceinline__ void step(const Args &a, uint32_t i, int key, float t, float p) {
+    if (i > 0 && !(kp < key || (kp == key && (tp < t || (tp == t && pp <= p))))) bad = true;
+    if ((i == 0 || kp != key) && key < a.nkeys) a.key_first[key] = i + 1u;  // its (sector, row) begins here
     kp = key;
     tp = t;
     pp = p;
@@ -202,7 +155,7 @@ __device__ __forceinline__ void stage_quantize(const Args &a, int vec, uint32_t 
     for (int e = 0; e < 8; ++e) {
       const int sec = (int)((sw[e >> 1] >> (16 * (e & 1))) & 0xffffu), row = (int)((rw[e >> 1] >> (16 * (e & 1))) & 0xffffu);
       const int key = sec * kNRows + row;
-      ck.step(key, tv[e], pv[e], i0 + e == 0);
+      ck.step(a, i0 + e, key, tv[e], pv[e]);
       q[e] = quant_checked(sec, row, pv[e], tv[e], nsect, ck.bad);
     }
     int4 *dst = reinterpret_cast<int4 *>(a.tq + i0);
@@ -217,20 +170,33 @@ __device__ __forceinline__ void stage_quantize(const Args &a, int vec, uint32_t 
       ck.tp = a.time[i - 1];
       ck.pp = a.pad[i - 1];
     }
-    ck.step(sec * kNRows + row, t, p, i == 0);
+    ck.step(a, i, sec * kNRows + row, t, p);
     a.tq[i] = quant_checked(sec, row, p, t, nsect, ck.bad);
   }
   if (ck.bad) raise(a.ctr, kErrInput);
 }
 
 #ifndef TPC_STAGES_ONLY
-__global__ void __launch_bounds__(256) k_quantize(Args a, int vec) { stage_quantize(a, vec, blockIdx.x, gridDim.x); }
+// The last CTA to finish builds the tables: with a pass of its own (a binary search per
+// key, then the same table) the ingest of a 0.9 M frame took 18 us more.
+__global__ void __launch_bounds__(256) k_quantize(Args a, int vec) {
+  pdl_begin();
+  stage_quantize(a, vec, blockIdx.x, gridDim.x);
+  __shared__ bool s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(&a.ctr[kCtrIndexDone], 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  stage_row_index_table(a);
+}
 
 void launch_quantize(const Args &a, int sms, cudaStream_t st) {
   const bool vec = ((((uintptr_t)a.pad | (uintptr_t)a.time | (uintptr_t)a.sector | (uintptr_t)a.row) & 15) == 0);
   const uint32_t blocks = (a.n / 8 + 255) / 256 + 1;
   const uint32_t cap = (uint32_t)sms * 8u;
-  k_quantize<<<blocks < cap ? blocks : cap, 256, 0, st>>>(a, vec ? 1 : 0);
+  launch_pdl(k_quantize, blocks < cap ? blocks : cap, 256, 0, st, a.n, a, vec ? 1 : 0);
 }
 
 // The neighbour kernels' fixed-point conversion, element by element (tests of
@@ -242,12 +208,6 @@ __global__ void __launch_bounds__(256) k_debug_quantize(const float *__restrict_
 void launch_debug_quantize(const float *v, uint32_t n, int32_t *q, cudaStream_t st) {
   const uint32_t blocks = (n + 255) / 256;
   k_debug_quantize<<<blocks < 8192u ? blocks : 8192u, 256, 0, st>>>(v, n, q);
-}
-
-void launch_row_index(const Args &a, cudaStream_t st) {
-  const int warps = a.nkeys + 1;
-  const int blocks = (warps * 32 + 255) / 256;
-  k_row_index<<<blocks, 256, 0, st>>>(a);
 }
 
 #endif  // TPC_STAGES_ONLY

@@ -119,6 +119,7 @@ struct __align__(16) ListSmem {
 static_assert(sizeof(ListSmem) <= 48 * 1024, "static shared memory");
 
 __global__ void __launch_bounds__(kPruneWarps * 32) k_prune(Args a, const MlpW *__restrict__ W, float logit_tau) {
+  pdl_begin();
   __shared__ ListSmem sm;
   const uint32_t n_amb = min(a.ctr[kCtrAmb], a.amb_cap);
   if (blockIdx.x * kPruneWarps >= n_amb) return;  // the whole block has nothing to do
@@ -459,6 +460,7 @@ __global__ void __launch_bounds__(256, 4) k_mlp_score_tc(const MlpW *__restrict_
                                                          const float *__restrict__ feat, uint32_t m,
                                                          const uint32_t *__restrict__ m_dev,
                                                          float *__restrict__ logit, int *err) {
+  pdl_begin();
   if (m_dev) m = min(m, *m_dev);
   extern __shared__ __align__(1024) unsigned char smraw[];
   TcMlpSmem &sm = *reinterpret_cast<TcMlpSmem *>(smraw);
@@ -538,6 +540,7 @@ __global__ void __launch_bounds__(kPruneWarps * 32) k_mlp_score(const MlpW *__re
                                                                 const float *__restrict__ feat, uint32_t m,
                                                                 const uint32_t *__restrict__ m_dev,
                                                                 float *__restrict__ logit) {
+  pdl_begin();
   if (m_dev) m = min(m, *m_dev);  // (as in k_mlp_score_tc)
   __shared__ PruneSmem sm;
   stage_weights(sm, W);
@@ -677,6 +680,7 @@ __device__ __forceinline__ int nth_from_top(uint32_t m, int n) {
 
 __global__ void __launch_bounds__(kRegionThreads, kRegionCtasPerSm)
     k_region_feat(Args a, float *__restrict__ feat, int4 *__restrict__ meta, int64_t *__restrict__ cost) {
+  pdl_begin();
   __shared__ int s_rec[kRegionGroup + 1], s_row[kRegionGroup];
   __shared__ uint32_t s_base;
   __shared__ uint32_t s_warp[kRegionThreads / 32];
@@ -757,6 +761,7 @@ __global__ void __launch_bounds__(kRegionThreads, kRegionCtasPerSm)
 __global__ void __launch_bounds__(256) k_region_decide(Args a, const float *__restrict__ logit,
                                                        const int4 *__restrict__ meta, const int64_t *__restrict__ cost,
                                                        uint32_t rows_cap, float logit_tau) {
+  pdl_begin();
   const uint32_t m = min(a.ctr[kCtrRegionRows], rows_cap);
   uint32_t clusters = 0;
   for (uint32_t d = blockIdx.x * blockDim.x + threadIdx.x; d < m; d += gridDim.x * blockDim.x) {
@@ -787,18 +792,19 @@ void launch_region_rescore(const Args &a, const MlpW *w, const MlpHead &head, fl
                            int64_t *cost, float *logit, float logit_tau, int sms, int engine,
                            cudaStream_t st) {
   const uint32_t rows_cap = a.tile_cap * (uint32_t)kPruneRegionRows;
-  k_region_feat<<<sms * 2 * kRegionCtasPerSm, kRegionThreads, 0, st>>>(a, feat, meta, cost);
+  launch_pdl(k_region_feat, (uint32_t)(sms * 2 * kRegionCtasPerSm), kRegionThreads, 0, st, a.n, a, feat, meta, cost);
   const uint32_t *m_dev = a.ctr + kCtrRegionRows;
   if (engine == TPC_MMA_SYNC)
-    k_mlp_score<<<sms * 8, kPruneWarps * 32, 0, st>>>(w, feat, rows_cap, m_dev, logit);
+    launch_pdl(k_mlp_score, (uint32_t)sms * 8u, kPruneWarps * 32, 0, st, a.n, w, feat, rows_cap, m_dev, logit);
   else  // 4 CTAs per SM, as in launch_mlp_score_tc
-    k_mlp_score_tc<<<sms * 4, 256, mlp_score_tc_smem(), st>>>(w, head, feat, rows_cap, m_dev, logit,
-                                                               reinterpret_cast<int *>(a.ctr + kCtrErr));
-  k_region_decide<<<sms * 8, 256, 0, st>>>(a, logit, meta, cost, rows_cap, logit_tau);
+    launch_pdl(k_mlp_score_tc, (uint32_t)sms * 4u, 256, mlp_score_tc_smem(), st, a.n, w, head, feat, rows_cap, m_dev, logit,
+               reinterpret_cast<int *>(a.ctr + kCtrErr));
+  launch_pdl(k_region_decide, (uint32_t)sms * 8u, 256, 0, st, a.n, a, logit, meta, cost, rows_cap, logit_tau);
 }
 
 void launch_prune(const Args &a, const MlpW *w, float logit_tau, int sms, cudaStream_t st) {
-  k_prune<<<sms * 5, kPruneWarps * 32, 0, st>>>(a, w, logit_tau);  // 5 CTAs per SM: its registers and shared memory allow 5
+  // 5 CTAs per SM: its registers and shared memory allow 5
+  launch_pdl(k_prune, (uint32_t)sms * 5u, kPruneWarps * 32, 0, st, a.n, a, w, logit_tau);
 }
 
 void launch_mlp_pack(const float *theta, const float *mean, const float *inv_std, MlpW *w, cudaStream_t st) {

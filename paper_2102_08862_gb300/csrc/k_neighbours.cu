@@ -450,23 +450,34 @@ __device__ __forceinline__ void stage_tile_windows(const Args &a, uint32_t bid, 
     if (r >= 1 && r <= kNRows - 2 && tb > ta) {
       const int t0 = a.tq[ta].x, t1 = a.tq[tb - 1].x;
       const int pb = a.row_begin[key - 1], pe = rb, nb = re, ne = a.row_begin[key + 2];
-      // the four lower bounds (first e in [lo, hi) with t_q(e) >= x) advance
-      // together, so that their loads are in flight at once; a finished search
-      // keeps loading its own position (< n: the array is padded) and ignores it
+      // the four lower bounds (first e in [lo, hi) with t_q(e) >= x) advance together
+      // and quarter their ranges, so that twelve loads are in flight at once and the
+      // dependent round trips are half those of halving; a finished search keeps
+      // loading its own position (< n: the array is padded) and ignores it
       int lo[4] = {pb, pb, nb, nb}, hi[4] = {pe, pe, ne, ne};
       const int x[4] = {t0 - a.wt, t1 + a.wt + 1, t0 - a.wt, t1 + a.wt + 1};
       for (;;) {
         bool more = false;
-        int tm[4], mid[4];
+        int m[4][3], tm[4][3];
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
-          mid[s] = (int)(((unsigned)lo[s] + (unsigned)hi[s]) >> 1);
-          tm[s] = a.tq[mid[s]].x;
+          const int len = max(hi[s] - lo[s], 0);  // (probes lo <= m0 <= m1 <= m2 < hi)
+          m[s][0] = lo[s] + (len >> 2);
+          m[s][1] = lo[s] + (len >> 1);
+          m[s][2] = lo[s] + (len >> 1) + (len >> 2);
+#pragma unroll
+          for (int p = 0; p < 3; ++p) tm[s][p] = a.tq[m[s][p]].x;
         }
 #pragma unroll
         for (int s = 0; s < 4; ++s)
           if (lo[s] < hi[s]) {
-            if (tm[s] < x[s]) lo[s] = mid[s] + 1; else hi[s] = mid[s];
+            if (tm[s][1] < x[s]) {
+              if (tm[s][2] < x[s]) lo[s] = m[s][2] + 1;
+              else lo[s] = m[s][1] + 1, hi[s] = m[s][2];
+            } else {
+              if (tm[s][0] < x[s]) lo[s] = m[s][0] + 1, hi[s] = m[s][1];
+              else hi[s] = m[s][0];
+            }
             more |= lo[s] < hi[s];
           }
         if (!more) break;
@@ -581,6 +592,7 @@ __device__ __forceinline__ void nb_tile(const Args &a, int win_cap, uint32_t t, 
 template <bool kPrune, int TILE, int CAP, int THREADS>
 __global__ void __launch_bounds__(THREADS, THREADS == 128 ? 10 : 5)
     k_neighbours(Args a, int win_cap) {
+  pdl_begin();
   const uint32_t t = blockIdx.x;
   if (t >= min(a.ctr[kCtrTiles], a.tile_cap)) return;
   uint32_t phase = 0;
@@ -608,7 +620,7 @@ __device__ __forceinline__ void stage_neighbours(const Args &a, int win_cap, uin
 // smallest (cost_i, i); a row-151 cluster k takes as down link the row-150
 // cluster i with up[i] = k of smallest (cost_i, i).  The claimants lie inside
 // j's (k's) time window, so the kernel scans that window of the adjacent row and
-// recomputes each claimant's triplet cost exactly.  grid.y = 72 edge rows.
+// recomputes each claimant's triplet cost exactly.
 constexpr int kClaimBlocks = 32;  // blocks per edge row
 __device__ __forceinline__ void edge_claims_block(const Args &a, int e, int x) {
   const int s = e >> 1;
@@ -649,21 +661,27 @@ __device__ __forceinline__ void stage_edge_claims(const Args &a, uint32_t bid, u
 }
 
 #ifndef TPC_STAGES_ONLY
-__global__ void __launch_bounds__(256) k_tile_windows(Args a) { stage_tile_windows(a, blockIdx.x, gridDim.x); }
-__global__ void __launch_bounds__(256) k_edge_claims(Args a) { edge_claims_block(a, blockIdx.y, blockIdx.x); }
+__global__ void __launch_bounds__(256) k_tile_windows(Args a) {
+  pdl_begin();
+  stage_tile_windows(a, blockIdx.x, gridDim.x);
+}
+__global__ void __launch_bounds__(256) k_edge_claims(Args a) {
+  pdl_begin();
+  edge_claims_block(a, (int)blockIdx.x / kClaimBlocks, (int)blockIdx.x % kClaimBlocks);
+}
 
 // ------------------------------------------------------------------ launchers
 void launch_tile_windows(const Args &a, cudaStream_t st) {
   const uint32_t tiles = neighbour_tiles_max(a.n, a.nkeys, a.nb_tile);
-  k_tile_windows<<<(tiles + 255) / 256, 256, 0, st>>>(a);
+  launch_pdl(k_tile_windows, (tiles + 255) / 256, 256, 0, st, a.n, a);
 }
 
 template <int TILE, int CAP, int THREADS>
 static void launch_nb(const Args &a, int row_cap, cudaStream_t st, bool prune) {
   const int cap = row_cap > 0 && row_cap < CAP - 1 ? row_cap : CAP - 1;
   const uint32_t grid = neighbour_tiles_max(a.n, a.nkeys, TILE);
-  if (prune) k_neighbours<true, TILE, CAP, THREADS><<<grid, THREADS, 0, st>>>(a, cap);
-  else k_neighbours<false, TILE, CAP, THREADS><<<grid, THREADS, 0, st>>>(a, cap);
+  launch_pdl(prune ? k_neighbours<true, TILE, CAP, THREADS> : k_neighbours<false, TILE, CAP, THREADS>, grid, THREADS, 0, st,
+             a.n, a, cap);
 }
 
 void launch_neighbours(const Args &a, int row_cap, int sms, cudaStream_t st, bool prune) {
@@ -674,7 +692,7 @@ void launch_neighbours(const Args &a, int row_cap, int sms, cudaStream_t st, boo
 }
 
 void launch_edge_claims(const Args &a, cudaStream_t st) {
-  k_edge_claims<<<dim3(kClaimBlocks, 2 * a.nsect), 256, 0, st>>>(a);
+  launch_pdl(k_edge_claims, (uint32_t)(kClaimBlocks * 2 * a.nsect), 256, 0, st, a.n, a);
 }
 #endif  // TPC_STAGES_ONLY
 

@@ -5,8 +5,8 @@
 // device functions that take the block index and the number of blocks; this
 // file includes those sources without their kernels and launchers and runs the
 // stages in one kernel, one after the other, with a grid-wide barrier between
-// stages that depend on each other: validation and quantisation together with
-// the (sector, row) keys; the tile table (one block); the tile windows; the
+// stages that depend on each other: validation and quantisation with the (sector,
+// row) begins; the row index and tile table (one block); the tile windows; the
 // neighbours; the edge-row claims; the mutual links and start hits; the start
 // list; the chain walk; the cluster_track assignment together with the Kalman fit.
 // The grid is as many CTAs as fit on the GPU at once, so that every CTA is resident; each
@@ -73,7 +73,6 @@ template <int TILE, int CAP>
 __global__ void __launch_bounds__(256, 6) k_track_persistent(Args a, int vec, int win_cap) {
   const uint32_t bid = blockIdx.x, nblk = gridDim.x;
   stage_quantize(a, vec, bid, nblk);
-  stage_row_index_keys(a, bid, nblk);
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
   if (bid == 0) stage_row_index_table(a);
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
@@ -90,7 +89,7 @@ __global__ void __launch_bounds__(256, 6) k_track_persistent(Args a, int vec, in
   stage_walk<false>(a, bid);
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
   stage_assign<0>(a, bid, nblk, nullptr);  // (reads the chains, as the fit does: no barrier between them)
-  stage_fit(a, bid, nblk);
+  stage_fit<256>(a, bid, nblk);
 }
 
 int g_pers_blocks[64][3];  // [device][tile variant]: resident CTAs per SM (0: not yet known)

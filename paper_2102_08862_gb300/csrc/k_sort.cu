@@ -95,6 +95,7 @@ static_assert(sizeof(BinLarge) <= 232448, "shared memory of one CTA");
 __global__ void __launch_bounds__(kChunkThreads) k_sort_count(Args a, const uint16_t *__restrict__ sector,
                                                               const uint16_t *__restrict__ row, SortScratch s,
                                                               uint32_t chunk) {
+  pdl_begin();
   __shared__ int32_t h[kBins];
   __shared__ uint32_t s_warp[kChunkThreads / 32];
   __shared__ bool s_last;
@@ -145,6 +146,7 @@ __global__ void __launch_bounds__(kChunkThreads) k_sort_scatter(Args a, const ui
                                                                 const float *__restrict__ pad,
                                                                 const float *__restrict__ time, SortScratch s,
                                                                 uint32_t chunk, float4 *__restrict__ rec) {
+  pdl_begin();
   __shared__ int32_t cur[kBins];
   const int32_t *base = s.base + (size_t)blockIdx.x * kBinStride;
   for (int k = threadIdx.x; k < kBins; k += kChunkThreads) cur[k] = s.offset[k] + base[k];  // (unused where the chunk has none)
@@ -303,6 +305,7 @@ __global__ void __launch_bounds__(THREADS) k_sort_bins(Args a, const float4 *__r
                                                        const uint16_t *__restrict__ row, uint16_t *s_sector,
                                                        uint16_t *s_row, float *s_pad, float *s_time, int32_t *perm,
                                                        SortScratch s) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char smraw[];
   auto &sm = *reinterpret_cast<BinSmem<CAP, BUCKETS> *>(smraw);
   if constexpr (CAP == kCapSmall) {
@@ -349,11 +352,14 @@ int launch_sort(const Args &a, const uint16_t *sector, const uint16_t *row, cons
   if (a.n == 0) return 1;
   const uint32_t chunks = sort_chunks(a.n), chunk = (a.n + chunks - 1) / chunks;
   float4 *rec = static_cast<float4 *>(records);
-  k_sort_count<<<chunks, kChunkThreads, 0, st>>>(a, sector, row, s, chunk);
-  k_sort_scatter<<<chunks, kChunkThreads, 0, st>>>(a, sector, row, pad, time, s, chunk, rec);
-  small<<<kBins, 256, sizeof(BinSmall), st>>>(a, rec, sector, row, s_sector, s_row, s_pad, s_time, perm, s);
-  mid<<<2 * sms, 1024, sizeof(BinMid), st>>>(a, rec, sector, row, s_sector, s_row, s_pad, s_time, perm, s);
-  large<<<sms, 1024, sizeof(BinLarge), st>>>(a, rec, sector, row, s_sector, s_row, s_pad, s_time, perm, s);
+  launch_pdl(k_sort_count, chunks, kChunkThreads, 0, st, a.n, a, sector, row, s, chunk);
+  launch_pdl(k_sort_scatter, chunks, kChunkThreads, 0, st, a.n, a, sector, row, pad, time, s, chunk, rec);
+  launch_pdl(small, (uint32_t)kBins, 256, sizeof(BinSmall), st, a.n, a, rec, sector, row, s_sector, s_row, s_pad, s_time,
+             perm, s);
+  launch_pdl(mid, 2u * (uint32_t)sms, 1024, sizeof(BinMid), st, a.n, a, rec, sector, row, s_sector, s_row, s_pad, s_time, perm,
+             s);
+  launch_pdl(large, (uint32_t)sms, 1024, sizeof(BinLarge), st, a.n, a, rec, sector, row, s_sector, s_row, s_pad, s_time, perm,
+             s);
   return 6;
 }
 

@@ -70,10 +70,15 @@ size_t carve(unsigned char *base, uint32_t n, uint32_t list_cap, Args *a, size_t
     return p;
   };
   const size_t tiles_l = link_tiles(n), tiles_k = walk_tiles(n);
-  *reset_bytes = kNCounters * 4 + 8 * (tiles_l + tiles_k);
+  // the start list and mask need less than the 4 bytes per cluster counted here; the
+  // keys' first clusters live on the difference, so that the frames that fit stay the same
+  const size_t keys = up256(reset_words(kNKeys) * 4) - up256(kNCounters * 4), starts_room = up256(((size_t)n / 2 + 2) * 8);
+  const size_t starts_need = start_bits_offset(n) + ((size_t)n / 32 + 1) * 4;
+  *reset_bytes = reset_words(kNKeys) * 4 + 8 * (tiles_l + tiles_k);
   unsigned char *reset = take(*reset_bytes);
   a->ctr = reinterpret_cast<uint32_t *>(reset);
-  a->lb_links = reinterpret_cast<uint64_t *>(reset ? reset + kNCounters * 4 : nullptr);
+  a->key_first = a->ctr ? a->ctr + kNCounters : nullptr;
+  a->lb_links = reinterpret_cast<uint64_t *>(a->ctr ? a->ctr + reset_words(kNKeys) : nullptr);
   a->lb_keep = a->lb_links ? a->lb_links + tiles_l : nullptr;
   a->row_begin = reinterpret_cast<int32_t *>(take((kNKeys + 1) * 4));
   a->tile_off = reinterpret_cast<int32_t *>(take((kNKeys + 1) * 4));
@@ -85,7 +90,7 @@ size_t carve(unsigned char *base, uint32_t n, uint32_t list_cap, Args *a, size_t
   a->link = reinterpret_cast<int2 *>(take(((size_t)n + 4) * 8));
   a->tq = reinterpret_cast<int2 *>(take(((size_t)n + 8) * 8));
   a->mup16 = reinterpret_cast<uint16_t *>(take(((size_t)n + 16) * 2));
-  unsigned char *starts = take(starts_bytes(n));
+  unsigned char *starts = take(starts_room > keys + starts_need ? starts_room - keys : starts_need);
   a->starts = reinterpret_cast<int32_t *>(starts);
   a->start_bits = reinterpret_cast<uint32_t *>(starts ? starts + start_bits_offset(n) : nullptr);
   a->trk_key = reinterpret_cast<int32_t *>(take(((size_t)list_cap + 1) * 4));
@@ -176,7 +181,6 @@ extern "C" int tpc_track_timeframe_noalloc(const tpc_tf_config *cfg, const tpc_c
   if (cudaMemsetAsync(a.ctr, 0, reset_bytes, st) != cudaSuccess)
     return report(TPC_ERR_CUDA, "tpc_track_timeframe_noalloc: clearing the counters failed");
   launch_quantize(a, sms, st);
-  launch_row_index(a, st);
   launch_tile_windows(a, st);
   launch_neighbours(a, 0, sms, st);
   launch_edge_claims(a, st);

@@ -106,6 +106,7 @@ struct Args {
   const float *time;
   const int32_t *perm;     // sorted position -> caller index, nullptr for identity
   int2 *tq;                // [n + 8] quantised (t_q, y_q) of every sorted cluster (written by the ingest pass)
+  uint32_t *key_first;     // [nkeys] index + 1 of each (sector, row)'s first cluster (reset to 0)
   int32_t *row_begin;      // [kNKeys + 1]
   int32_t *tile_off;       // [kNKeys + 1] first neighbour tile of each (sector, row)
   int4 *tile_win;          // per tile: candidate ranges in rows r-1 and r+1 (lo, hi, lo, hi)
@@ -202,6 +203,17 @@ __device__ __forceinline__ uint16_t ld_keep_u16(const uint16_t *addr, uint64_t p
 }
 __device__ __forceinline__ void st_keep_u16(uint16_t *addr, uint16_t v, uint64_t pol) {
   asm volatile("st.global.L2::cache_hint.u16 [%0], %1, %2;" ::"l"(addr), "h"(v), "l"(pol) : "memory");
+}
+
+// ------------------------------------------------- launch overlap
+// The kernels of a call are launched so that each may begin while its predecessor
+// still runs (launch_pdl): its first statement waits until the predecessor has
+// finished and its results are visible.  Every CTA waits, so that a finished kernel
+// means that all before it have finished too.  Then the next kernel's CTAs may be
+// placed as soon as all of this one's have started.
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // ------------------------------------------------- block scan

@@ -31,8 +31,35 @@ inline size_t walk_tiles(uint32_t n) { return (n / 2 + 1 + kWalkTileN - 1) / kWa
 // upper bound of neighbour tiles for n clusters
 inline uint32_t neighbour_tiles_max(uint32_t n, int nkeys, int tile) { return n / (uint32_t)tile + (uint32_t)nkeys + 1; }
 
-void launch_row_index(const Args &a, cudaStream_t st);
-// validation of every sorted cluster and its quantised (t, y) into a.tq
+// Launch of a kernel that begins with pdl_begin(), in a call with n clusters: up to
+// kOverlapMax of them it may be placed while the kernel before it on the stream still
+// runs (programmatic stream serialisation), which hides the gap between two dependent
+// kernels.  A call, us: 0.9 M clusters 245 -> 215, 6.2 M 402 -> 400; but 11 M 570 -> 577,
+// 32 M 1559 -> 1650: blocks placed early, where the predecessor's end, bunch on a few
+// SMs.  The arguments are converted to the kernel's.
+constexpr uint32_t kOverlapMax = 4u << 20;
+template <class... P, class... A>
+inline void launch_pdl(void (*kernel)(P...), uint32_t grid, uint32_t block, size_t smem, cudaStream_t st, uint32_t n,
+                       A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = n <= kOverlapMax ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// 32-bit words at the head of the per-call reset region: the counters, then key_first
+// (an even number: the 8-byte look-back words follow)
+inline size_t reset_words(int nkeys) { return (size_t)kNCounters + (((size_t)nkeys + 1) & ~(size_t)1); }
+
+// validation of every sorted cluster, its quantised (t, y) into a.tq, the (sector, row)
+// index and the tile table
 void launch_quantize(const Args &a, int sms, cudaStream_t st);
 void launch_tile_windows(const Args &a, cudaStream_t st);
 // prune = true also lists the clusters with >= 2 pairs under the cost cut in a.amb
@@ -48,10 +75,13 @@ void launch_first_list(const Args &a, int sms, cudaStream_t st);
 void launch_walk(const Args &a, int sms, cudaStream_t st);
 // cluster_track, one (sector, row) per CTA step: -1, then each crossing track's id
 void launch_assign(const Args &a, int sms, cudaStream_t st);
-// opts the assignment kernel in to its 48 KB of shared memory (0 on success)
+// opts the kernels that hold the assignment in to its 48 KB of shared memory (0 on success)
 int assign_prepare();
+int fit_assign_prepare();
 void launch_debug_links(const Args &a, int32_t *mup, uint8_t *is_start, cudaStream_t st);
 void launch_fit(const Args &a, int sms, int variant, cudaStream_t st);
+// the thread-per-track fit and the assignment in one launch
+void launch_fit_assign(const Args &a, int sms, cudaStream_t st);
 // track follower: pick-ups, claims and join proposals (k_follow); the joined
 // paths numbered and fitted into the caller's records (k_follow_fit); then
 // cluster_track rewritten with the new ids (k_follow_ct)
