@@ -1341,9 +1341,8 @@ extern "C" int tpc_tf_remove_unassigned(tpc_tf *tf, const tpc_clusters *cl, cons
   cudaStream_t st = (cudaStream_t)stream;
   Args a;
   fill_args(tf, n, nullptr, a);
-  // the compaction's counters and look-back words (the error word stays)
-  TPC_CK(cudaMemsetAsync(tf->reset + kCtrCompactTile, 0, 8, st));
-  TPC_CK(cudaMemsetAsync(a.lb_links, 0, 8 * link_tiles(n), st));
+  // the compaction's counter (the error word stays)
+  TPC_CK(cudaMemsetAsync(tf->reset + kCtrCompactTile, 0, 4, st));
   launch_compact(a, cl->sector, cl->row, cl->pad, cl->time, cluster_track, sector, row, pad, time, track, count,
                  tf->sms, st);
   TPC_CK(cudaGetLastError());

@@ -31,8 +31,7 @@ namespace tpc {
 
 namespace {
 constexpr int kThreads = 256;
-constexpr int kItems = kLinkTileN / kThreads;    // clusters per thread of a hit-removal tile
-constexpr int kLinkTile = kThreads * kItems;     // clusters per look-back tile of the hit removal
+constexpr int kLinkTile = kLinkTileN;  // clusters per tile of the hit removal
 constexpr uint16_t kNone16 = 0xffff;
 
 }  // namespace
@@ -330,102 +329,134 @@ __global__ void __launch_bounds__(kThreads) k_assign(Args a) {
   stage_assign<kAssignCap>(a, blockIdx.x, gridDim.x, assign_buf);
 }
 
-// Hit removal: the clusters attached to a track, in caller order (an ordered
-// compaction over 2048-cluster tiles taken in order from a counter, with a
-// decoupled look-back across tiles).  Inputs and outputs are in caller order.
-// Thread t of a tile holds elements t + 256 q (q = 0..7), so every load is
-// coalesced; positions inside the tile come from warp ballots per q and one scan
-// of the 64 (q, warp) counts (the element order is q-major, then warp, then
-// lane); the kept clusters are staged in shared memory at their tile positions
-// and written out coalesced.
+// Hit removal: the clusters attached to a track, in caller order.  k_compact_count
+// counts the kept ones of every 2048-cluster tile (4 B per cluster), its last CTA turns
+// the counts into offsets; k_compact then copies each tile on its own: a warp holds 256
+// consecutive clusters, 32 at a time, so that loads are coalesced and the kept ones of a
+// round go to consecutive places.  No tile waits for another.
+// What bounds it: memory, 4 + 16 B per cluster and 16 per kept one.  16.8 M clusters, 90
+// % kept: 0.125 ms (k_compact 0.086, 5.8 TB/s).  An ordered compaction in one pass (each tile's fields loaded once a
+// look-back had told its place, staged in shared memory) took 0.183 ms.
+__global__ void __launch_bounds__(kThreads) k_compact_count(uint32_t n, const int32_t *__restrict__ ct, int vec,
+                                                            uint32_t *__restrict__ offset, uint32_t *o_count,
+                                                            uint32_t *ctr) {
+  __shared__ uint32_t s_warp[kThreads / 32];
+  __shared__ bool s_last;
+  const uint32_t n_tiles = (n + kLinkTile - 1) / kLinkTile;
+  const uint32_t lane = threadIdx.x & 31;
+  for (uint32_t tile = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); tile < n_tiles;
+       tile += gridDim.x * (kThreads / 32)) {  // a tile per warp
+    const uint32_t i0 = tile * kLinkTile;
+    uint32_t c = 0;
+    if (vec && i0 + kLinkTile <= n) {
+      const int4 *p = reinterpret_cast<const int4 *>(ct + i0) + lane;
+#pragma unroll 8
+      for (int q = 0; q < kLinkTile / 128; ++q) {
+        const int4 x = p[32 * q];
+        c += (x.x >= 0) + (x.y >= 0) + (x.z >= 0) + (x.w >= 0);
+      }
+    } else {
+      for (uint32_t i = i0 + lane; i < min(n, i0 + kLinkTile); i += 32) c += ct[i] >= 0;
+    }
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (lane == 0) offset[tile] = c;
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(&ctr[kCtrCompactTile], 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  // exclusive scan: each thread's tiles in turn, kScan read at a time
+  constexpr uint32_t kScan = 32;
+  const uint32_t per = (n_tiles + kThreads - 1) / kThreads;
+  const uint32_t t0 = min(n_tiles, threadIdx.x * per), t1 = min(n_tiles, t0 + per);
+  uint32_t sum = 0, total;
+  for (uint32_t t = t0; t < t1; t += kScan) {
+    uint32_t v[kScan];
+#pragma unroll
+    for (uint32_t u = 0; u < kScan; ++u) v[u] = t + u < t1 ? __ldcg(offset + t + u) : 0u;
+#pragma unroll
+    for (uint32_t u = 0; u < kScan; ++u) sum += v[u];
+  }
+  uint32_t run = block_exclusive_scan<kThreads>(sum, s_warp, &total);
+  for (uint32_t t = t0; t < t1; t += kScan) {
+    uint32_t v[kScan];
+#pragma unroll
+    for (uint32_t u = 0; u < kScan; ++u) v[u] = t + u < t1 ? __ldcg(offset + t + u) : 0u;
+#pragma unroll
+    for (uint32_t u = 0; u < kScan; ++u) {
+      if (t + u < t1) offset[t + u] = run;
+      run += v[u];
+    }
+  }
+  if (threadIdx.x == 0) *o_count = total;
+}
+
 __global__ void __launch_bounds__(kThreads) k_compact(uint32_t n, const uint16_t *__restrict__ sector,
                                                       const uint16_t *__restrict__ row, const float *__restrict__ pad,
                                                       const float *__restrict__ time, const int32_t *__restrict__ ct,
-                                                      uint16_t *o_sector, uint16_t *o_row, float *o_pad,
-                                                      float *o_time, int32_t *o_track, uint32_t *o_count,
-                                                      uint64_t *lb, uint32_t *ctr, uint32_t spin_limit) {
-  constexpr int kWarps = kThreads / 32;
-  static_assert(kItems * kWarps == 64, "two (q, warp) counts per lane of the scanning warp");
-  __shared__ uint32_t s_tile, s_prefix, s_total;
-  __shared__ uint32_t s_cnt[kItems * kWarps];  // kept per (q, warp), then their offsets
-  __shared__ uint16_t s_sec[kLinkTile], s_row[kLinkTile];
-  __shared__ float s_pad[kLinkTile], s_time[kLinkTile];
-  __shared__ int32_t s_trk[kLinkTile];
-  const uint32_t n_tiles = (n + kLinkTile - 1) / kLinkTile;
+                                                      const uint32_t *__restrict__ offset,
+                                                      uint16_t *__restrict__ o_sector, uint16_t *__restrict__ o_row,
+                                                      float *__restrict__ o_pad, float *__restrict__ o_time,
+                                                      int32_t *__restrict__ o_track) {
+  constexpr int kWarps = kThreads / 32, kRounds = kLinkTile / kThreads;
+  __shared__ uint32_t s_cnt[kWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (;;) {
-    if (threadIdx.x == 0) s_tile = atomicAdd(&ctr[kCtrCompactTile], 1u);
-    __syncthreads();
-    const uint32_t tile = s_tile;
-    if (tile >= n_tiles) break;
-    const uint32_t base = tile * kLinkTile;
-    int32_t t[kItems];
-    uint32_t mask[kItems];
+  const uint32_t i0 = blockIdx.x * kLinkTile + (uint32_t)warp * (kRounds * 32u) + (uint32_t)lane;
+  int32_t t[kRounds];
+  uint16_t sec[kRounds], rw[kRounds];
+  float p[kRounds], tm[kRounds];
 #pragma unroll
-    for (int q = 0; q < kItems; ++q) {
-      const uint32_t i = base + threadIdx.x + q * kThreads;
-      t[q] = i < n ? __ldcs(ct + i) : -1;
-      mask[q] = __ballot_sync(0xffffffffu, t[q] >= 0);
-      if (lane == 0) s_cnt[q * kWarps + warp] = (uint32_t)__popc(mask[q]);
+  for (int q = 0; q < kRounds; ++q) {
+    const uint32_t i = i0 + 32u * (uint32_t)q;
+    t[q] = -1;
+    if (i < n) {
+      t[q] = __ldcs(ct + i);
+      sec[q] = __ldcs(sector + i);
+      rw[q] = __ldcs(row + i);
+      p[q] = __ldcs(pad + i);
+      tm[q] = __ldcs(time + i);
     }
-    __syncthreads();
-    if (warp == 0) {  // exclusive scan of the 64 counts in element order, then the look-back
-      const uint32_t v0 = s_cnt[lane], v1 = s_cnt[lane + 32];
-      uint32_t x0 = v0, x1 = v1;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y0 = __shfl_up_sync(0xffffffffu, x0, o), y1 = __shfl_up_sync(0xffffffffu, x1, o);
-        if (lane >= o) {
-          x0 += y0;
-          x1 += y1;
-        }
-      }
-      const uint32_t half = __shfl_sync(0xffffffffu, x0, 31);
-      s_cnt[lane] = x0 - v0;
-      s_cnt[lane + 32] = half + x1 - v1;
-      const uint32_t total = half + __shfl_sync(0xffffffffu, x1, 31);
-      const uint32_t pre = lookback_exclusive(lb, tile, total, ctr, spin_limit);
-      if (lane == 0) {
-        s_prefix = pre;
-        s_total = total;
-      }
-    }
-    __syncthreads();
-    const uint32_t below = (1u << lane) - 1u;
-#pragma unroll
-    for (int q = 0; q < kItems; ++q)
-      if (t[q] >= 0) {
-        const uint32_t i = base + threadIdx.x + q * kThreads;
-        const uint32_t p = s_cnt[q * kWarps + warp] + (uint32_t)__popc(mask[q] & below);
-        s_sec[p] = sector[i];
-        s_row[p] = row[i];
-        s_pad[p] = pad[i];
-        s_time[p] = time[i];
-        s_trk[p] = t[q];
-      }
-    __syncthreads();
-    const uint32_t total = s_total, out0 = s_prefix;
-    for (uint32_t k = threadIdx.x; k < total; k += kThreads) {
-      o_sector[out0 + k] = s_sec[k];
-      o_row[out0 + k] = s_row[k];
-      o_pad[out0 + k] = s_pad[k];
-      o_time[out0 + k] = s_time[k];
-      if (o_track) o_track[out0 + k] = s_trk[k];
-    }
-    if (tile == n_tiles - 1 && threadIdx.x == 0) *o_count = out0 + total;
-    __syncthreads();
   }
-  if (n == 0 && blockIdx.x == 0 && threadIdx.x == 0) *o_count = 0;
+  uint32_t mask[kRounds], mine = 0;
+#pragma unroll
+  for (int q = 0; q < kRounds; ++q) {
+    mask[q] = __ballot_sync(0xffffffffu, t[q] >= 0);
+    mine += (uint32_t)__popc(mask[q]);
+  }
+  if (lane == 0) s_cnt[warp] = mine;
+  __syncthreads();
+  uint32_t pos = offset[blockIdx.x];
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w)
+    if (w < warp) pos += s_cnt[w];
+  const uint32_t below = (1u << lane) - 1u;
+#pragma unroll
+  for (int q = 0; q < kRounds; ++q) {
+    if (t[q] >= 0) {
+      const uint32_t o = pos + (uint32_t)__popc(mask[q] & below);
+      o_sector[o] = sec[q];
+      o_row[o] = rw[q];
+      o_pad[o] = p[q];
+      o_time[o] = tm[q];
+      if (o_track) o_track[o] = t[q];
+    }
+    pos += (uint32_t)__popc(mask[q]);
+  }
 }
 
 void launch_compact(const Args &a, const uint16_t *sector, const uint16_t *row, const float *pad, const float *time,
                     const int32_t *ct, uint16_t *o_sector, uint16_t *o_row, float *o_pad, float *o_time,
                     int32_t *o_track, uint32_t *o_count, int sms, cudaStream_t st) {
-  const uint32_t tiles = (a.n + kLinkTile - 1) / kLinkTile;
-  // 6 CTAs per SM fit (40 registers, 33 KB of shared memory each)
-  const uint32_t grid = tiles < (uint32_t)sms * 6u ? (tiles ? tiles : 1u) : (uint32_t)sms * 6u;
-  k_compact<<<grid, kThreads, 0, st>>>(a.n, sector, row, pad, time, ct, o_sector, o_row, o_pad, o_time, o_track,
-                                       o_count, a.lb_links, a.ctr, a.spin_limit);
+  const uint32_t tiles = (a.n + kLinkTile - 1) / kLinkTile, cap = (uint32_t)sms * 8u;
+  uint32_t *offset = reinterpret_cast<uint32_t *>(a.lb_links);  // (a word per tile; no look-back here)
+  const uint32_t blocks = (tiles + kThreads / 32 - 1) / (kThreads / 32);
+  k_compact_count<<<blocks < cap ? (blocks ? blocks : 1u) : cap, kThreads, 0, st>>>(
+      a.n, ct, ((uintptr_t)ct & 15) == 0 ? 1 : 0, offset, o_count, a.ctr);
+  if (tiles > 0)
+    k_compact<<<tiles, kThreads, 0, st>>>(a.n, sector, row, pad, time, ct, offset, o_sector, o_row, o_pad, o_time,
+                                          o_track);
 }
 
 // inspection: the mutual up link as a sorted position, and the start flag

@@ -73,8 +73,7 @@ enum : int {
   kCtrTiles = 9,    // neighbour tiles of this frame
   kCtrAmb = 10,     // clusters listed for the separate rescoring kernel (pruned mode)
   kCtrQueued = 11,  // clusters rescored from the tile regions (pruned mode)
-  kCtrCompactTile = 12,  // hit removal: next tile
-  kCtrCompactKept = 13,  // hit removal: clusters kept
+  kCtrCompactTile = 12,  // hit removal: counting CTAs that have finished
   kCtrFollowTile = 14,   // track follower: next track to follow
   kCtrFollowTracks = 15, // track follower: tracks after joining
   kCtrFollowPathTile = 16,  // track follower: next tile of joined paths
@@ -121,7 +120,7 @@ struct Args {
   uint16_t *trk_rl;        // [track list capacity] first row | chain length << 8 (the assignment pass)
   uint32_t *sec_first;     // [nsect] smallest track id of each sector (~0u: none), reset by the row index
   uint32_t *sec_cnt;       // [nsect] tracks of each sector
-  uint64_t *lb_links;      // look-back words of the start list and of the hit removal, one per 2048 clusters
+  uint64_t *lb_links;      // look-back words of the start list (the hit removal keeps its tiles' offsets here), one per 2048 clusters
   uint64_t *lb_keep;       // look-back words, one per 1024-start tile
   uint32_t *ctr;           // counters (kNCounters)
   uint32_t starts_cap;
