@@ -644,17 +644,17 @@ __device__ int32_t fol_member(const Args &a, uint32_t R, int k) {
 
 }  // namespace
 
-// Tiles of 256 chain tracks in order: the roots of the tile are numbered by a
+// Tiles of kFollowTileN chain tracks in order: the roots of the tile are numbered by a
 // block scan and a decoupled look-back; each root's thread counts its path,
 // locates its middle and last members, and runs the tracklet fit over the path
 // (the same seed and filter as k_fit_thread, transported across row gaps); the
 // new id of every track on the path goes to map for the cluster pass.
-__global__ void __launch_bounds__(256) k_follow_fit(Args a) {
+__global__ void __launch_bounds__(kFollowTileN) k_follow_fit(Args a) {
   __shared__ uint32_t s_tile, s_prefix;
-  __shared__ uint32_t s_warp[8];
-  __shared__ uint32_t s_key[256], s_excl[256];
+  __shared__ uint32_t s_warp[kFollowTileN / 32];
+  __shared__ uint32_t s_key[kFollowTileN], s_excl[kFollowTileN];
   const uint32_t nt = min(a.ctr[kCtrTracks], a.track_list_cap);
-  const uint32_t n_tiles = (nt + 255) / 256;
+  const uint32_t n_tiles = (nt + kFollowTileN - 1) / kFollowTileN;
   if (n_tiles == 0) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       a.ctr[kCtrFollowTracks] = 0;
@@ -667,10 +667,10 @@ __global__ void __launch_bounds__(256) k_follow_fit(Args a) {
     __syncthreads();
     const uint32_t tile = s_tile;
     if (tile >= n_tiles) break;
-    const uint32_t R = tile * 256 + threadIdx.x;
+    const uint32_t R = tile * kFollowTileN + threadIdx.x;
     const bool root = R < nt && a.fl.pred[R] == kFolNone;
     uint32_t total;
-    const uint32_t excl = block_exclusive_scan<256>(root ? 1u : 0u, s_warp, &total);
+    const uint32_t excl = block_exclusive_scan<kFollowTileN>(root ? 1u : 0u, s_warp, &total);
     if (threadIdx.x < 32) {
       const uint32_t pre = lookback_exclusive(a.fl.lb, tile, total, a.ctr, a.spin_limit);
       if (threadIdx.x == 0) s_prefix = pre;
@@ -704,7 +704,7 @@ __global__ void __launch_bounds__(256) k_follow_fit(Args a) {
     s_key[threadIdx.x] = root ? ((uint32_t)Lr << 9) | (1u << 8) | threadIdx.x : threadIdx.x;
     s_excl[threadIdx.x] = excl;
     __syncthreads();
-    for (int k2 = 2; k2 <= 256; k2 <<= 1)
+    for (int k2 = 2; k2 <= kFollowTileN; k2 <<= 1)
       for (int j = k2 >> 1; j > 0; j >>= 1) {
         const int i = threadIdx.x, ixj = i ^ j;
         if (ixj > i) {
@@ -719,7 +719,7 @@ __global__ void __launch_bounds__(256) k_follow_fit(Args a) {
     const uint32_t key = s_key[threadIdx.x];
     if (key & (1u << 8)) {
       const uint32_t src = key & 255u;
-      const uint32_t R = tile * 256 + src;
+      const uint32_t R = tile * kFollowTileN + src;
       const uint32_t id = s_prefix + s_excl[src];
       const int L = (int)(key >> 9);
       if (id < a.track_capacity) {
@@ -791,7 +791,7 @@ __global__ void __launch_bounds__(256) k_follow_fit(Args a) {
   }
 }
 
-void launch_follow_fit(const Args &a, int sms, cudaStream_t st) { k_follow_fit<<<sms * 8, 256, 0, st>>>(a); }
+void launch_follow_fit(const Args &a, int sms, cudaStream_t st) { k_follow_fit<<<sms * (2048 / kFollowTileN), kFollowTileN, 0, st>>>(a); }
 
 #endif  // TPC_STAGES_ONLY
 

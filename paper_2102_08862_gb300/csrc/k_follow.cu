@@ -791,7 +791,9 @@ __global__ void __launch_bounds__(kThreads) k_time_samples(Args a) {
 
 void launch_follow(const Args &a, int sms, cudaStream_t st) {
   k_time_samples<<<sms * 4, kThreads, 0, st>>>(a);
-  k_follow<<<sms * 4, kThreads, 0, st>>>(a);
+  // a lane for every track of a 5 ms frame: 4 CTAs per SM (all that are resident) gave some
+  // lanes two tracks, 0.394 ms; 6 or more, 0.337
+  k_follow<<<sms * 8, kThreads, 0, st>>>(a);
 }
 
 void launch_follow_ct(const Args &a, int sms, cudaStream_t st) { k_follow_ct<<<sms * 8, kThreads, 0, st>>>(a); }

@@ -91,10 +91,11 @@ void launch_follow_ct(const Args &a, int sms, cudaStream_t st);
 // cross-sector links of the followed tracks into a.fl.next (a.fl.pred reset to ~0
 // before; a.fl.succ is reused)
 void launch_sector_links(const Args &a, int sms, cudaStream_t st);
-// look-back tiles of the follower (256 tracks each) for n clusters
+// look-back tiles of the follower (kFollowTileN tracks each, 256 at most) for n clusters
+constexpr int kFollowTileN = 128;
 inline size_t follow_tiles(uint32_t n, int n_min, uint32_t track_list_cap) {
   const size_t nt = (size_t)n / (size_t)(n_min > 0 ? n_min : 1) + 1;
-  return ((nt < track_list_cap ? nt : track_list_cap) + 255) / 256 + 1;
+  return ((nt < track_list_cap ? nt : track_list_cap) + kFollowTileN - 1) / kFollowTileN + 1;
 }
 // unsorted input: stable sort by (sector, row, time, pad) into the sorted views
 // (records: 16 bytes per cluster, free again when the sort is done)
