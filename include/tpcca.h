@@ -194,7 +194,7 @@ int tpc_track_timeframe(tpc_tf *tf, const tpc_clusters *cl, const tpc_tracks *ou
  * records back and synchronises the stream.  cluster_track is copied back on an
  * internal stream of the handle as soon as it is final (while the fit runs).  A
  * sorted frame of at least 4 Mi clusters (without cross-sector links) whose host
- * arrays are all page-locked goes through as three sector ranges whose copies in,
+ * arrays are all page-locked goes through as two to four sector ranges whose copies in,
  * tracking and copies back overlap; the results are those of the one-piece call.
  * out->n_tracks and out->n_tracks_host are host pointers here (either may be NULL). */
 int tpc_track_timeframe_host(tpc_tf *tf, const tpc_clusters *cl, const tpc_tracks *out, void *stream);
@@ -251,8 +251,7 @@ int tpc_tf_autotune(tpc_tf *tf, const tpc_clusters *cl, const tpc_tracks *out, i
  * device arrays with room for cl->n entries; cl->flags is ignored (inputs in
  * caller order).  Uses the handle's scratch: enqueue it on the stream of the
  * tracking call, after it.  Errors: TPC_ERR_ARG, TPC_ERR_CAPACITY (n >
- * max_clusters), TPC_ERR_CUDA; a bounded wait that gave up surfaces through
- * tpc_tf_status. */
+ * max_clusters), TPC_ERR_CUDA. */
 int tpc_tf_remove_unassigned(tpc_tf *tf, const tpc_clusters *cl, const int32_t *cluster_track, uint16_t *sector,
                              uint16_t *row, float *pad, float *time, int32_t *track, uint32_t *count, void *stream);
 

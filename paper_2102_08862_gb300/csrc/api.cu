@@ -41,7 +41,10 @@ int fail(int code, const std::string &msg) {
 constexpr int kMaxStages = 12;
 constexpr int kMaxRanges = 8;             // sector ranges of a pipelined host-buffer call
 constexpr uint32_t kRangeMinClusters = 1u << 22;  // smaller frames are copied in one piece
-constexpr int kRanges = 3;  // measured on the 10 ms frame: 3 ranges 7.45e9 clusters/s end to end, 4: 7.30e9, 6: 6.66e9, 8: 6.15e9
+// Sector ranges of a pipelined call: more overlap more of the copies, but each pays the
+// latency of a call.  Measured, us a call with 2 / 3 / 4 ranges: 5 M clusters 987 / 1120 /
+// 1298; 16.8 M 2108 / 2132 / 2169; 32 M 3667 / 3350 / 3284.
+int host_ranges(uint32_t n) { return n < (16u << 20) ? 2 : n < (24u << 20) ? 3 : 4; }
 
 constexpr int kPinnedCounters = 32;  // (of the 64 words of the handle's page-locked buffer)
 static_assert(kPinnedCounters + kNCounters <= 64, "page-locked words");
@@ -954,9 +957,9 @@ extern "C" int tpc_track_timeframe_host(tpc_tf *tf, const tpc_clusters *cl, cons
   cudaStream_t st = (cudaStream_t)stream;
   // large sorted frames without cross-sector links, in page-locked buffers:
   // pipelined over sector ranges
-  if ((cl->flags & TPC_INPUT_SORTED) && tf->cfg.follow != 2 && n >= kRangeMinClusters && tf->nsect >= kRanges &&
+  if ((cl->flags & TPC_INPUT_SORTED) && tf->cfg.follow != 2 && n >= kRangeMinClusters && tf->nsect >= host_ranges(n) &&
       host_arrays_pinned(cl, out))
-    return track_host_ranges(tf, cl, out, st, kRanges);
+    return track_host_ranges(tf, cl, out, st, host_ranges(n));
   if (n > 0) {
     TPC_CK(cudaMemcpyAsync(tf->h_sector, cl->sector, (size_t)n * 2, cudaMemcpyHostToDevice, st));
     TPC_CK(cudaMemcpyAsync(tf->h_row, cl->row, (size_t)n * 2, cudaMemcpyHostToDevice, st));
