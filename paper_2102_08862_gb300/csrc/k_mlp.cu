@@ -341,7 +341,7 @@ struct __align__(1024) TcMlpSmem {
   unsigned char w1[64 * 16 * 2];      // W1 (N 64, K 16)
   unsigned char w2[64 * 64 * 2];      // W2 (N 64, K 64)
   unsigned char wb2[64 * 16 * 2];     // b2 as three BF16 parts in K columns 12..14 (N 64, K 16), else 0
-  uint64_t mbar;
+  uint64_t mbar[2];
   uint32_t tmem;
 };
 
@@ -392,6 +392,19 @@ __device__ __forceinline__ void tc_fold_b1(TcMlpSmem &sm, const MlpW *__restrict
   }
 }
 
+// barriers of one warpgroup of the dense scorer (0 is the CTA's)
+__device__ __forceinline__ void wg_sync(int h) { asm volatile("barrier.cta.sync %0, 128;" ::"r"(1 + h) : "memory"); }
+__device__ __forceinline__ bool wg_and(int h, bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.and.pred q, %2, 128, p;\n selp.u32 %0, 1, 0, "
+      "q;\n}\n"
+      : "=r"(r)
+      : "r"((uint32_t)v), "r"(1 + h)
+      : "memory");
+  return r != 0;
+}
+
 // first-layer epilogue with the bias already in Z1: ReLU and BF16 only
 __device__ __forceinline__ void tc_epi_hidden_nb(uint32_t lane_addr, unsigned char *hb, int hr) {
   uint32_t z[32];
@@ -413,18 +426,17 @@ __device__ __forceinline__ void tc_epi_hidden_nb(uint32_t lane_addr, unsigned ch
 // bank (operands of the FP32 instructions themselves: no shared-memory loads)
 __device__ __forceinline__ float tc_epi_logit_c(uint32_t lane_addr, const MlpHead &hd) {
   float z[16];
-  float acc0 = hd.b3, acc1 = 0.f;
+  float2 acc = make_float2(hd.b3, 0.f);  // even and odd units
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     tc_ld16(lane_addr + 16u * q, z);
     tc_wait_ld();
 #pragma unroll
-    for (int c = 0; c < 16; c += 2) {  // Z2 holds b2 already
-      acc0 = fmaf(fmaxf(z[c], 0.f), hd.w3[16 * q + c], acc0);
-      acc1 = fmaf(fmaxf(z[c + 1], 0.f), hd.w3[16 * q + c + 1], acc1);
-    }
+    for (int c = 0; c < 16; c += 2)  // Z2 holds b2 already
+      acc = __ffma2_rn(make_float2(fmaxf(z[c], 0.f), fmaxf(z[c + 1], 0.f)),
+                       make_float2(hd.w3[16 * q + c], hd.w3[16 * q + c + 1]), acc);
   }
-  return acc0 + acc1;
+  return acc.x + acc.y;
 }
 
 // row r of the tile at x: standardised BF16 inputs, then 1, 1, 1 (the bias columns), 0
@@ -447,13 +459,15 @@ __device__ __forceinline__ void tc_put_input_c(unsigned char *x, int r, const fl
 }
 
 // logits of raw feature rows (float[m][12]) on the tcgen05 path.  A CTA of 256
-// threads takes two 128-row tiles per step: warpgroup h (threads 128 h ..) holds
-// tile h, thread r of it row r (tensor-memory lane r, columns 64 h ..).  Both
-// tiles' MMAs of a layer are issued together and complete behind one mbarrier
-// wait; the next step's row is loaded while the current step runs.  4 CTAs share
-// an SM (tensor memory: 4 x 128 of 512 columns; 64 registers a thread), 32 warps
-// in all, which hide the MMA and load latencies; the per-row constants are kernel
-// parameters (MlpHead), so the epilogues read no shared memory.
+// threads holds two 128-row tiles, warpgroup h (threads 128 h ..) tile h, thread r of it
+// row r (tensor-memory lane r, columns 64 h ..).  The warpgroups share the staged
+// weights only: each issues its own MMAs, waits on its own mbarrier and meets at its own
+// named barrier, so that one's epilogue runs while the other's MMAs do (5.2 M rows: both
+// tiles in step 111.1 us, so 109.9; with the output layer's multiply-adds one by one
+// instead of in pairs 113.4).  The next step's row is loaded while the current step runs.  4 CTAs share an SM (tensor memory: 4 x 128 of
+// 512 columns; 64 registers a thread), 32 warps in all, which hide the MMA and load
+// latencies; the per-row constants are kernel parameters (MlpHead), so the epilogues
+// read no shared memory.
 // With m_dev set, the rows are the first min(*m_dev, m) (a count written on the
 // device by an earlier kernel of the stream; m is then the buffers' capacity).
 __global__ void __launch_bounds__(256, 4) k_mlp_score_tc(const MlpW *__restrict__ W, const __grid_constant__ MlpHead hd,
@@ -468,16 +482,20 @@ __global__ void __launch_bounds__(256, 4) k_mlp_score_tc(const MlpW *__restrict_
   tc_stage_weights(sm, W);
   __syncthreads();  // the bias columns overwrite part of the staged W1 rows
   tc_fold_b1(sm, W);
-  if (tid == 0) mbar_init(&sm.mbar, 1);
+  if (tid == 0) {
+    mbar_init(&sm.mbar[0], 1);
+    mbar_init(&sm.mbar[1], 1);
+  }
   if (warp == 0) tc_alloc(&sm.tmem, 128);
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = sm.tmem;
-  const uint32_t lane_addr = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + 64u * (uint32_t)h;
+  const uint32_t tmem = sm.tmem, acc = tmem + 64u * (uint32_t)h;
+  const uint32_t lane_addr = acc + ((uint32_t)(32 * (warp & 3)) << 16);
   const uint32_t steps = (m + 255) / 256;
   const uint32_t idesc = tc_idesc_bf16(128, 64);
+  uint64_t *mbar = &sm.mbar[h];
   float f[kMlpIn];
   if (blockIdx.x < steps) load_feature_row(feat, blockIdx.x * 256 + 128 * h + r, m, f);
   bool ok = true;
@@ -485,50 +503,40 @@ __global__ void __launch_bounds__(256, 4) k_mlp_score_tc(const MlpW *__restrict_
     const uint32_t row = u * 256 + 128 * h + r;
     tc_put_input_c(sm.x[h], r, f, row < m, hd);
     if (u + gridDim.x < steps) load_feature_row(feat, (u + gridDim.x) * 256 + 128 * h + r, m, f);  // next step
-    // layer 1: X (128 x 16) W1^T of both tiles (b1 included)
+    // layer 1: X (128 x 16) W1^T (b1 included)
     fence_async_smem();
     tc_fence_before();
-    __syncthreads();
+    wg_sync(h);
     tc_fence_after();
-    if (tid == 0) {
-#pragma unroll
-      for (int t = 0; t < 2; ++t)
-        tc_mma_bf16(tmem + 64u * t, tc_desc(smem_u32(sm.x[t]), 128, 256), tc_desc(smem_u32(sm.w1), 128, 256), idesc,
-                    false);
-      tc_commit(&sm.mbar);
+    if (r == 0) {
+      tc_mma_bf16(acc, tc_desc(smem_u32(sm.x[h]), 128, 256), tc_desc(smem_u32(sm.w1), 128, 256), idesc, false);
+      tc_commit(mbar);
     }
-    ok = __all_sync(0xffffffffu, mbar_wait(&sm.mbar, 0, 1u << 22));  // warp-uniform (tcgen05.ld)
+    ok = __all_sync(0xffffffffu, mbar_wait(mbar, 0, 1u << 22));  // warp-uniform (tcgen05.ld)
     tc_fence_after();
     if (ok) tc_epi_hidden_nb(lane_addr, sm.h[h], r);
     fence_async_smem();
     tc_fence_before();
-    ok = __syncthreads_and(ok);  // layer 2 only if every thread saw layer 1 complete
+    ok = wg_and(h, ok);  // layer 2 only if every thread saw layer 1 complete
     tc_fence_after();
     if (!ok) break;
-    // layer 2: b2 (X against the parts of b2), then H1 (128 x 64) W2^T in four K = 16
-    // steps, for both tiles
-    if (tid == 0) {
-      const uint32_t w0 = smem_u32(sm.w2);
+    // layer 2: b2 (X against the parts of b2), then H1 (128 x 64) W2^T in four K = 16 steps
+    if (r == 0) {
+      const uint32_t w0 = smem_u32(sm.w2), h0 = smem_u32(sm.h[h]);
+      tc_mma_bf16(acc, tc_desc(smem_u32(sm.x[h]), 128, 256), tc_desc(smem_u32(sm.wb2), 128, 256), idesc, false);  // b2
 #pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        const uint32_t h0 = smem_u32(sm.h[t]);
-        tc_mma_bf16(tmem + 64u * t, tc_desc(smem_u32(sm.x[t]), 128, 256), tc_desc(smem_u32(sm.wb2), 128, 256), idesc,
-                    false);  // b2
-#pragma unroll
-        for (int k4 = 0; k4 < 4; ++k4)
-          tc_mma_bf16(tmem + 64u * t, tc_desc(h0 + 256 * k4, 128, 1024), tc_desc(w0 + 256 * k4, 128, 1024), idesc,
-                      true);
-      }
-      tc_commit(&sm.mbar);
+      for (int k4 = 0; k4 < 4; ++k4)
+        tc_mma_bf16(acc, tc_desc(h0 + 256 * k4, 128, 1024), tc_desc(w0 + 256 * k4, 128, 1024), idesc, true);
+      tc_commit(mbar);
     }
-    ok = __all_sync(0xffffffffu, mbar_wait(&sm.mbar, 1, 1u << 22));
+    ok = __all_sync(0xffffffffu, mbar_wait(mbar, 1, 1u << 22));
     tc_fence_after();
     const float lg = ok ? tc_epi_logit_c(lane_addr, hd) : 0.f;
     tc_fence_before();
-    ok = __syncthreads_and(ok);  // sm.x, sm.h and the accumulators are free again
+    ok = wg_and(h, ok);  // sm.x, sm.h and the accumulator are free again
     if (ok && row < m) logit[row] = lg;
   }
-  if (!ok && tid == 0) atomicOr(err, (int)kErrTimeout);
+  if (!ok && r == 0) atomicOr(err, (int)kErrTimeout);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tc_dealloc(tmem, 128);
