@@ -210,9 +210,10 @@ __device__ __forceinline__ void st_keep_u16(uint16_t *addr, uint16_t v, uint64_t
 // finished and its results are visible.  Every CTA waits, so that a finished kernel
 // means that all before it have finished too.  Then the next kernel's CTAs may be
 // placed as soon as all of this one's have started.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_trigger();
 }
 
 // ------------------------------------------------- block scan

@@ -66,6 +66,7 @@ __global__ void __launch_bounds__(kTrWarps * 32) k_train_fwd_bwd(const float *__
                                                                  const int32_t *__restrict__ idx, uint32_t B,
                                                                  const MlpW *__restrict__ W, float pos_weight,
                                                                  float inv_B, float *__restrict__ partial) {
+  pdl_trigger();
   extern __shared__ __align__(16) unsigned char smraw[];
   TrainSmem &sm = *reinterpret_cast<TrainSmem *>(smraw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
@@ -363,6 +364,7 @@ __global__ void __launch_bounds__(kTcTrRows, 2) k_train_fwd_bwd_tc(const float *
                                                                const MlpW *__restrict__ W, float pos_weight,
                                                                float inv_B, float *__restrict__ partial,
                                                                uint32_t *__restrict__ err) {
+  pdl_trigger();
   extern __shared__ __align__(1024) unsigned char smraw_[];
   TrainTcSmem &sm = *reinterpret_cast<TrainTcSmem *>(
       (reinterpret_cast<uintptr_t>(smraw_) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -674,9 +676,11 @@ __global__ void k_train_update(const float *__restrict__ partial, int nparts, fl
                                float *__restrict__ m1, float *__restrict__ m2, MlpW *__restrict__ W,
                                float *__restrict__ grad_out, float *__restrict__ loss_out, float lr, float beta1,
                                float beta2, float eps, float bc1, float bc2, int do_update) {
+  pdl_begin();
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p > kMlpNParam) return;
   float gsum = 0.f;
+#pragma unroll 16  // (loads in flight; the order of the sum is fixed)
   for (int c = 0; c < nparts; ++c) gsum += partial[(size_t)c * kPartStride + p];
   if (p == kMlpNParam) {
     if (loss_out) *loss_out = gsum;
@@ -812,9 +816,10 @@ int launch_step(tpc_mlp_trainer *tr, const float *feat, const uint8_t *label, co
     bc1 = (float)(1.0 - std::pow((double)tr->cfg.beta1, tr->step));
     bc2 = (float)(1.0 - std::pow((double)tr->cfg.beta2, tr->step));
   }
-  k_train_update<<<(kMlpNParam + 1 + 255) / 256, 256, 0, st>>>(tr->partial, parts, tr->theta, tr->m1, tr->m2, tr->w,
-                                                               grad, loss, tr->cfg.lr, tr->cfg.beta1, tr->cfg.beta2,
-                                                               tr->cfg.eps, bc1, bc2, update ? 1 : 0);
+  // placed while the partial gradients are computed (n = 0: always); 64 threads a block,
+  // so that the loads of the partials come from 80 SMs
+  launch_pdl(k_train_update, (uint32_t)(kMlpNParam + 1 + 63) / 64u, 64, 0, st, 0u, tr->partial, parts, tr->theta, tr->m1,
+             tr->m2, tr->w, grad, loss, tr->cfg.lr, tr->cfg.beta1, tr->cfg.beta2, tr->cfg.eps, bc1, bc2, update ? 1 : 0);
   TR_CK(cudaGetLastError());
   return TPC_OK;
 }
