@@ -83,8 +83,12 @@ __global__ void __launch_bounds__(256, 6) k_track_persistent(Args a, int vec, in
   stage_edge_claims(a, bid, nblk);
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
   stage_links(a, bid, nblk);
-  if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
-  stage_start_list(a);
+  if (one_tile_list(a.n)) {
+    stage_last_list(a, nblk);
+  } else {
+    if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
+    stage_start_list(a);
+  }
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
   stage_walk<false>(a, bid);
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
