@@ -23,8 +23,8 @@
 //    are numbered in the order of their ids; every member gets the new id; the
 //    tracks are fitted again over their clusters (rows may be skipped).
 //
-// GB300 design: in k_follow each lane follows one track at a time and takes the
-// next from a counter, one row per pass of its loop whichever direction it is
+// GB300 design: in k_follow each lane follows one track at a time and goes on
+// to its next one (grid stride), one row per pass of its loop whichever direction it is
 // in, so the lanes of a warp stay busy and together although follows differ in
 // length.  Candidates of a row are found by a search of its time-sorted
 // clusters (binary over every 16th time, kept apart so that it stays in L2, then

@@ -343,9 +343,10 @@ __global__ void __launch_bounds__(kThreads) k_assign(Args a) {
 // the counts into offsets; k_compact then copies each tile on its own: a warp holds 256
 // consecutive clusters, 32 at a time, so that loads are coalesced and the kept ones of a
 // round go to consecutive places.  No tile waits for another.
-// What bounds it: memory, 4 + 16 B per cluster and 16 per kept one.  16.8 M clusters, 90
-// % kept: 0.125 ms (k_compact 0.086, 5.8 TB/s).  An ordered compaction in one pass (each tile's fields loaded once a
-// look-back had told its place, staged in shared memory) took 0.183 ms.
+// What bounds it: memory, 4 + 16 B per cluster and 16 per kept one.  16.8 M clusters,
+// 90 % kept: 0.125 ms (k_compact 0.086, 5.8 TB/s).  An ordered compaction in one pass
+// (each tile's fields loaded once a look-back had told its place, staged in shared
+// memory) took 0.183 ms.
 __global__ void __launch_bounds__(kThreads) k_compact_count(uint32_t n, const int32_t *__restrict__ ct, int vec,
                                                             uint32_t *__restrict__ offset, uint32_t *o_count,
                                                             uint32_t *ctr) {

@@ -10,9 +10,9 @@
 // kernel writes a tile's ambiguous clusters into the tile's own region (their
 // candidates as two masks); k_region_feat enumerates their pairs into a dense
 // array of feature rows, the dense scorer (tcgen05 or mma.sync) scores it, and
-// k_region_decide decides each cluster from its contiguous rows.  Clusters that the neighbour kernel could not put in a region
-// (windows too large to stage, or the region full) are listed instead, and
-// k_prune rescores those: each warp takes 32 listed clusters and re-enumerates
+// k_region_decide decides each cluster from its contiguous rows.  Clusters that
+// the neighbour kernel could not put in a region (windows too large to stage, or
+// the region full) are listed instead, and k_prune rescores those: each warp takes 32 listed clusters and re-enumerates
 // their pairs from global memory.
 #include "mlp_dev.cuh"
 #include "tc_dev.cuh"

@@ -20,7 +20,7 @@
 // per lane.  Windows larger than the staging buffers are read from global memory
 // with the same arithmetic.
 //
-// What bounds it: instruction issue (82 % of the slots) and the integer pipe, which
+// What bounds it: instruction issue (79 % of the slots) and the integer pipe, which
 // takes half of them at half rate; DRAM traffic is 14 of the 16 bytes a cluster
 // needs, at a tenth of the bandwidth.  Warp instructions per 32 clusters (16.8 M
 // clusters, plain): staging 45, searches 66, scan 150, scoring and output 165.  In an

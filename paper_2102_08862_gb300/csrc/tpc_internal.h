@@ -34,8 +34,8 @@ inline uint32_t neighbour_tiles_max(uint32_t n, int nkeys, int tile) { return n 
 // Launch of a kernel that begins with pdl_begin(), in a call with n clusters: up to
 // kOverlapMax of them it may be placed while the kernel before it on the stream still
 // runs (programmatic stream serialisation), which hides the gap between two dependent
-// kernels.  A call, us: 0.9 M clusters 245 -> 215, 6.2 M 402 -> 400; but 11 M 570 -> 577,
-// 32 M 1559 -> 1650: blocks placed early, where the predecessor's end, bunch on a few
+// kernels.  A call, us: 0.9 M clusters 245 -> 213; but 11 M 570 -> 577, 16.8 M 780 -> 813,
+// 32 M 1632 -> 1708: blocks placed early, where the predecessor's end, bunch on a few
 // SMs.  The arguments are converted to the kernel's.
 constexpr uint32_t kOverlapMax = 4u << 20;
 template <class... P, class... A>
