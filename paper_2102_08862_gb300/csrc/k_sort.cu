@@ -14,7 +14,8 @@
 //      result does not depend on step 2's order.  A bin whose clusters crowd a bucket
 //      is sorted by a bitonic network instead.
 // A bin holds at most kSegCap clusters (more -> TPC_ERR_CAPACITY; pass sorted
-// input then).
+// input then).  The call goes on after that error, so a larger bin is filled too, with
+// an order of its own (fill_refused_bin).
 //
 // What bounds it: memory traffic, 4 B in per cluster for the count, 12 B in and 16 B
 // scattered out, 16 B in and 16 B out for the bins (0.06 ms for 6.2 M clusters at the
@@ -297,6 +298,27 @@ __device__ __forceinline__ void sort_bin(BinSmem<CAP, BUCKETS> &sm, const float4
   }
 }
 
+// A bin too large to sort: its clusters in the order of the records, so that the
+// permutation stays one (the later stages store through it), at coordinates that pass
+// the order check and cost the later stages little whatever the bin's size: times
+// spread over the whole validated range, pads beyond any window of the rows next to it.
+__device__ __forceinline__ void fill_refused_bin(const float4 *__restrict__ rec, int bin, int b, int cnt,
+                                                 const uint16_t *__restrict__ sector,
+                                                 const uint16_t *__restrict__ row, uint16_t *__restrict__ s_sector,
+                                                 uint16_t *__restrict__ s_row, float *__restrict__ s_pad,
+                                                 float *__restrict__ s_time, int32_t *__restrict__ perm) {
+  const float pad = bin & 1 ? 1000.0f : -1000.0f;  // (neighbouring rows: 2000 pads of 4 mm or more, wy < 4.2 m)
+  const float step = 196608.0f / (float)cnt;
+  for (int q = (int)threadIdx.x; q < cnt; q += (int)blockDim.x) {
+    const uint32_t i = __float_as_uint(rec[b + q].z);
+    perm[b + q] = (int32_t)i;
+    s_pad[b + q] = pad;
+    s_time[b + q] = fminf(fmaf((float)q, step, -65536.0f), 131072.0f);
+    s_sector[b + q] = bin < kNKeys ? (uint16_t)(bin / kNRows) : sector[i];
+    s_row[b + q] = bin < kNKeys ? (uint16_t)(bin % kNRows) : row[i];
+  }
+}
+
 // Every bin of up to kCapSmall clusters has a CTA of the small kernel; the larger
 // ones are taken from the lists by the middle and the large kernel's few CTAs.
 template <int CAP, int BUCKETS, int THREADS>
@@ -319,6 +341,7 @@ __global__ void __launch_bounds__(THREADS) k_sort_bins(Args a, const float4 *__r
       const int bin = s.list[m][e], b = s.offset[bin], cnt = s.offset[bin + 1] - b;
       if (cnt > CAP) {
         if (threadIdx.x == 0) raise(a.ctr, kErrSortCap);
+        fill_refused_bin(rec, bin, b, cnt, sector, row, s_sector, s_row, s_pad, s_time, perm);
         continue;
       }
       sort_bin<CAP, BUCKETS, THREADS>(sm, rec, bin, b, cnt, sector, row, s_sector, s_row, s_pad, s_time, perm);

@@ -1,0 +1,92 @@
+"""Input that a call refuses while its kernels run on: every store stays inside the
+caller's arrays, whatever an earlier frame left in the handle, and the next frame is
+tracked as ever."""
+import numpy as np
+import pytest
+
+import oracle as orc
+import tpcsynth as ts
+from gpu_util import as_dev, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+GUARD = 4096  # entries around cluster_track that no call may write
+MARK = -77
+
+
+@pytest.fixture(scope="module")
+def env():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2102_08862_gb300 import _build, tpcca
+    _build.build()
+    return tpcca, torch.device("cuda", 0)
+
+
+@pytest.fixture(scope="module")
+def frame():
+    f = ts.generate(ts.continuous(0.05, 11))
+    return f.sector, f.row, f.pad, f.time
+
+
+def _guarded_call(tpcca, dev, tr, arrays, sorted_input):
+    """One call with cluster_track between guards; (return code, cluster_track, first clusters)."""
+    import ctypes
+    d = as_dev(torch, dev, *arrays)
+    n = d[0].numel()
+    buf = torch.full((n + 2 * GUARD,), MARK, dtype=torch.int32, device=dev)
+    cnt = ctypes.c_uint32(0)
+    cl, out, _, cap = tr.structs(*d, sorted_input=sorted_input, host_count=cnt)
+    out.cluster_track = buf.data_ptr() + 4 * GUARD
+    rc = tpcca.tpc_track_timeframe(tr.handle, cl, out, torch.cuda.current_stream(dev).cuda_stream)
+    torch.cuda.synchronize()
+    guard = torch.cat([buf[:GUARD], buf[GUARD + n:]])
+    assert bool((guard == MARK).all()), "a store outside cluster_track"
+    m = min(cnt.value, cap)
+    return rc, buf[GUARD:GUARD + n].cpu().numpy(), tr._out["first_cluster"][:m].cpu().numpy(), cnt.value
+
+
+def _check_next_frame(tr, dev, frame):
+    ref = orc.track(*frame)
+    g = run_gpu(tr, torch, dev, *frame)
+    for name in ("down", "up", "mup"):
+        assert np.array_equal(g[name], ref[name]), name
+    assert np.array_equal(g["cluster_track"], ref["cluster_track"])
+
+
+def _crowd(keys, sizes, seed):
+    """Unsorted clusters, sizes[q] of them in (sector, row) keys[q]."""
+    rng = np.random.default_rng(seed)
+    key = np.repeat(keys, sizes)
+    n = key.size
+    p = rng.permutation(n)
+    return ((key // 152).astype(np.uint16)[p], (key % 152).astype(np.uint16)[p],
+            rng.uniform(0.0, 60.0, n).astype(np.float32), rng.uniform(0.0, 3000.0, n).astype(np.float32))
+
+
+@pytest.mark.parametrize("keys,sizes,code", [
+    ([40, 451], [16385, 5], "TPC_ERR_CAPACITY"),
+    ([40, 41, 42, 43], [20000, 17000, 16384, 30000], "TPC_ERR_CAPACITY"),  # neighbouring rows
+    ([40, 40 * 152 + 7], [500, 17000], "TPC_ERR_INPUT")])                  # sector 40
+@pytest.mark.parametrize("follow", [0, 2])
+def test_rows_beyond_the_sort(env, frame, keys, sizes, code, follow):
+    """More unsorted clusters of a (sector, row) than the sort holds, on a handle that has
+    tracked a larger unsorted frame of other rows."""
+    tpcca, dev = env
+    larger = [np.concatenate([a] * 6)[::-1] for a in frame]
+    larger[2] = larger[2] + np.repeat(np.arange(6, dtype=np.float32) * 2.0, len(frame[0]))
+    assert len(larger[0]) > sum(sizes)
+    tr = tpcca.TimeFrameTracker(len(larger[0]), follow=follow)
+    try:
+        tr.track(*as_dev(torch, dev, *larger), sorted_input=False)
+        bad = _crowd(keys, sizes, 5)
+        rc, ct, first, count = _guarded_call(tpcca, dev, tr, bad, False)
+        assert rc == getattr(tpcca, code)
+        assert ct.min() >= -1 and ct.max() < max(count, 1)  # every entry written
+        assert first.size == 0 or (first.min() >= 0 and first.max() < len(bad[0]))
+        if follow == 0:
+            _check_next_frame(tr, dev, frame)
+    finally:
+        tr.close()
