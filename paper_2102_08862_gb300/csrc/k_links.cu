@@ -161,6 +161,25 @@ __device__ __forceinline__ void stage_start_list(const Args &a) {
   stage_bit_list(a, a.starts, a.starts_cap, kCtrTileLinks, kCtrStarts);
 }
 
+// The (sector, row) of sorted position i: the last key with rb[key] <= i.  The links are
+// local to the rows of the positions, so a chain's keys come from there and not from the
+// input's sector and row, which invalid input has wrong (the chain would leave the row
+// table).  With rb in shared memory the search costs less than reading the two fields;
+// else the fields are tried first: two loads side by side against the search's chain.
+template <bool kSmemRb>
+__device__ __forceinline__ int key_at(const Args &a, const int32_t *rb, int i) {
+  if constexpr (!kSmemRb) {
+    const int k = min((int)a.sector[i] * kNRows + (int)a.row[i], a.nkeys - 1);
+    if (rb[k] <= i && i < rb[k + 1]) return k;
+  }
+  int lo = 0, hi = a.nkeys;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (rb[mid] <= i) lo = mid; else hi = mid;
+  }
+  return lo;
+}
+
 // A4: one start hit per thread (kWalkChains; walking two or four chains per
 // thread interleaved was slower: more threads hide the pointer chase better).
 // Chains that reach n_min clusters become tracks (ids in start order); their
@@ -182,7 +201,7 @@ __device__ __forceinline__ void stage_walk(const Args &a, uint32_t bid) {
   const int32_t *rb = a.row_begin;
   if constexpr (kSmemRb) {
     for (int k = threadIdx.x; k <= a.nkeys; k += kThreads) s_rb[k] = a.row_begin[k];
-    rb = s_rb;
+    rb = s_rb;  // (read behind the first barrier of the loop)
   }
   const int n_min = a.n_min;
   const size_t stride = a.track_list_cap;
@@ -211,7 +230,7 @@ __device__ __forceinline__ void stage_walk(const Args &a, uint32_t bid) {
       st[q] = make_int2(-1, 0);
       if (j + q < ns) {
         const int32_t i = a.starts[j + q];
-        st[q] = make_int2(i, min((int)a.sector[i] * kNRows + (int)a.row[i], a.nkeys - 1));
+        st[q] = make_int2(i, key_at<kSmemRb>(a, rb, i));
       }
       c[q] = st[q].x;
       kk[q] = st[q].y;

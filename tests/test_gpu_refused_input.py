@@ -90,3 +90,36 @@ def test_rows_beyond_the_sort(env, frame, keys, sizes, code, follow):
             _check_next_frame(tr, dev, frame)
     finally:
         tr.close()
+
+
+def _chain_heads(frame, count):
+    """First clusters of `count` tracks from the middle of a sorted frame."""
+    first = np.sort(orc.track(*frame)["tracks"]["first_cluster"])
+    first = first[(first > len(frame[0]) // 4) & (first < 3 * len(frame[0]) // 4)]
+    return first[:: max(1, len(first) // count)][:count]
+
+
+ENTRIES = {"handle": {}, "batched": dict(n_sectors=100), "persistent": dict(persistent=1), "followed": dict(follow=2)}
+
+
+@pytest.mark.parametrize("entry", list(ENTRIES))
+@pytest.mark.parametrize("field,value", [("sector", 200), ("sector", 65535), ("row", 180), ("row", 65535)])
+def test_chain_head_outside_the_detector(env, frame, entry, field, value):
+    """A sector or row that does not exist, on clusters that head a chain in the middle of
+    a sorted frame: the chain's links belong to the rows where the clusters lie."""
+    tpcca, dev = env
+    heads = _chain_heads(frame, 6)
+    assert len(heads) == 6
+    bad = [a.copy() for a in frame]
+    bad[("sector", "row").index(field)][heads] = value
+    tr = tpcca.TimeFrameTracker(len(frame[0]), **ENTRIES[entry])
+    try:
+        tr.track(*as_dev(torch, dev, *frame))
+        rc, ct, first, count = _guarded_call(tpcca, dev, tr, bad, True)
+        assert rc == tpcca.TPC_ERR_INPUT
+        assert ct.min() >= -1 and ct.max() < max(count, 1)
+        assert first.size == 0 or (first.min() >= 0 and first.max() < len(frame[0]))
+        if entry != "followed":
+            _check_next_frame(tr, dev, frame)
+    finally:
+        tr.close()
