@@ -18,6 +18,9 @@ namespace tpc {
 // keys, read at L2 (ld.cg: other blocks wrote them) kBatch at a time, so that one round
 // trip serves a whole frame's 22 keys per thread; block-wide scans join the blocks.
 // With unsorted input (an error) the minima keep row_begin monotone and inside [0, n].
+// The first key begins at 0 whatever it holds: clusters in front of the first one with a
+// valid key (an error too) lie in its row, so that every cluster is in a row and gets its
+// links written.
 __device__ __forceinline__ void stage_row_index_table(const Args &a) {
   constexpr int kBatch = 24;
   __shared__ int32_t s_min[256];
@@ -58,7 +61,7 @@ __device__ __forceinline__ void stage_row_index_table(const Args &a) {
 #pragma unroll
     for (int u = 0; u < kBatch; ++u)
       if (ke - 1 - u >= k0) {
-        const int32_t begin = v[u] ? min(run, (int32_t)v[u] - 1) : run;
+        const int32_t begin = ke - 1 - u == 0 ? 0 : v[u] ? min(run, (int32_t)v[u] - 1) : run;
         const int c = run - begin;
         a.row_begin[ke - 1 - u] = begin;
         mx = max(mx, c);

@@ -123,3 +123,49 @@ def test_chain_head_outside_the_detector(env, frame, entry, field, value):
             _check_next_frame(tr, dev, frame)
     finally:
         tr.close()
+
+
+@pytest.mark.parametrize("entry", ["handle", "persistent", "followed"])
+@pytest.mark.parametrize("bad", [1, 300, "all"])
+@pytest.mark.parametrize("sorted_input", [True, False])
+def test_frame_that_begins_outside_the_detector(env, frame, entry, bad, sorted_input):
+    """The first clusters, or all of them, in a sector that does not exist, on a handle
+    that has tracked a larger frame: they are in no row of the detector and link to nothing."""
+    tpcca, dev = env
+    larger = [np.concatenate([a] * 2)[::-1] for a in frame]
+    larger[2] = larger[2] + np.repeat(np.arange(2, dtype=np.float32) * 2.0, len(frame[0]))
+    n = len(frame[0])
+    b = [a.copy() for a in frame]
+    b[0][:n if bad == "all" else bad] = 40
+    tr = tpcca.TimeFrameTracker(len(larger[0]), **ENTRIES[entry])
+    try:
+        tr.track(*as_dev(torch, dev, *larger), sorted_input=False)
+        rc, ct, first, count = _guarded_call(tpcca, dev, tr, b, sorted_input)
+        assert rc == tpcca.TPC_ERR_INPUT
+        assert ct.min() >= -1 and ct.max() < max(count, 1)  # every entry written
+        assert bad != "all" or count == 0
+        assert first.size == 0 or (first.min() >= 0 and first.max() < n)
+        if entry != "followed":
+            _check_next_frame(tr, dev, frame)
+    finally:
+        tr.close()
+
+
+@pytest.mark.parametrize("bad", [1, 300, "all"])
+def test_noalloc_frame_that_begins_outside_the_detector(env, frame, bad):
+    tpcca, dev = env
+    import ctypes
+    n = len(frame[0])
+    b = [a.copy() for a in frame]
+    b[0][:n if bad == "all" else bad] = 40
+    tr = tpcca.TimeFrameTracker(n)  # (its output tensors)
+    try:
+        for arrays, code in ((frame, 0), (b, tpcca.TPC_ERR_INPUT), (frame, 0)):
+            cnt = ctypes.c_uint32(0)
+            d = as_dev(torch, dev, *arrays)
+            cl, out, _, _ = tr.structs(*d, host_count=cnt)
+            assert tpcca.tpc_track_timeframe_noalloc(None, cl, out, 0) == code
+        ref = orc.track(*frame)
+        assert np.array_equal(tr._out["cluster_track"][:n].cpu().numpy(), ref["cluster_track"])
+    finally:
+        tr.close()
