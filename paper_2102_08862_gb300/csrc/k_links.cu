@@ -161,25 +161,6 @@ __device__ __forceinline__ void stage_start_list(const Args &a) {
   stage_bit_list(a, a.starts, a.starts_cap, kCtrTileLinks, kCtrStarts);
 }
 
-// The (sector, row) of sorted position i: the last key with rb[key] <= i.  The links are
-// local to the rows of the positions, so a chain's keys come from there and not from the
-// input's sector and row, which invalid input has wrong (the chain would leave the row
-// table).  With rb in shared memory the search costs less than reading the two fields;
-// else the fields are tried first: two loads side by side against the search's chain.
-template <bool kSmemRb>
-__device__ __forceinline__ int key_at(const Args &a, const int32_t *rb, int i) {
-  if constexpr (!kSmemRb) {
-    const int k = min((int)a.sector[i] * kNRows + (int)a.row[i], a.nkeys - 1);
-    if (rb[k] <= i && i < rb[k + 1]) return k;
-  }
-  int lo = 0, hi = a.nkeys;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (rb[mid] <= i) lo = mid; else hi = mid;
-  }
-  return lo;
-}
-
 // A4: one start hit per thread (kWalkChains; walking two or four chains per
 // thread interleaved was slower: more threads hide the pointer chase better).
 // Chains that reach n_min clusters become tracks (ids in start order); their

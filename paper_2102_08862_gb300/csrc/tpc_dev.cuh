@@ -186,6 +186,27 @@ struct __align__(16) PruneRec {
 
 __device__ __forceinline__ int32_t caller_index(const Args &a, int32_t i) { return a.perm ? a.perm[i] : i; }
 
+// ------------------------------------------------- row of a position
+// The (sector, row) that sorted position i lies in: the last key with rb[key] <= i.
+// Links and windows are local to the rows of the positions, so the key that goes with
+// them comes from there and not from the input's sector and row, which invalid input has
+// wrong (it would lead out of the row table).  With rb in shared memory the search costs
+// less than reading the two fields; else the fields are tried first: two loads side by
+// side against the search's chain.
+template <bool kSmemRb>
+__device__ __forceinline__ int key_at(const Args &a, const int32_t *rb, int i) {
+  if constexpr (!kSmemRb) {
+    const int k = min((int)a.sector[i] * kNRows + (int)a.row[i], a.nkeys - 1);
+    if (rb[k] <= i && i < rb[k + 1]) return k;
+  }
+  int lo = 0, hi = a.nkeys;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (rb[mid] <= i) lo = mid; else hi = mid;
+  }
+  return lo;
+}
+
 // ------------------------------------------------- L2 residency hints
 // The 16-bit mutual links (2 B per cluster) are written by the link kernel and
 // chased by the walk: they are stored and loaded with an evict-last L2 policy,

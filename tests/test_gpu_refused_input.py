@@ -7,6 +7,7 @@ import pytest
 import oracle as orc
 import tpcsynth as ts
 from gpu_util import as_dev, run_gpu
+from mlp_util import random_net
 
 pytestmark = pytest.mark.gpu
 
@@ -167,5 +168,36 @@ def test_noalloc_frame_that_begins_outside_the_detector(env, frame, bad):
             assert tpcca.tpc_track_timeframe_noalloc(None, cl, out, 0) == code
         ref = orc.track(*frame)
         assert np.array_equal(tr._out["cluster_track"][:n].cpu().numpy(), ref["cluster_track"])
+    finally:
+        tr.close()
+
+
+@pytest.mark.parametrize("n_sectors", [36, 100])
+@pytest.mark.parametrize("field", ["sector", "row"])
+def test_listed_cluster_outside_the_detector(env, frame, field, n_sectors):
+    """Pruned mode, every window beyond the staging buffers, so that ambiguous clusters go
+    through the list; some of them have a sector or a row that does not exist."""
+    tpcca, dev = env
+    blob = tpcca.pack_blob(*random_net(6, feature_scale=True))
+    tr = tpcca.TimeFrameTracker(len(frame[0]), mode=tpcca.TPC_MODE_PRUNED, tau=0.5, row_cap=1, n_sectors=n_sectors)
+    try:
+        tr.load_mlp(blob)
+        tri = tr.extract(*as_dev(torch, dev, *frame))[2].cpu().numpy()
+        amb = np.unique(tri[:, 0])
+        amb = amb[len(amb) // 4:][:: max(1, len(amb) // 30)][:20]
+        assert len(amb) >= 10
+        bad = [a.copy() for a in frame]
+        bad[("sector", "row").index(field)][amb] = 65535
+        tr.track(*as_dev(torch, dev, *frame))
+        assert tr.pruned_split()[1] > 0
+        rc, ct, first, count = _guarded_call(tpcca, dev, tr, bad, True)
+        assert rc == tpcca.TPC_ERR_INPUT
+        assert tr.pruned_split()[1] > 0
+        assert ct.min() >= -1 and ct.max() < max(count, 1)
+        ref = orc.track(*frame, mlp=blob, tau=0.5)
+        g = run_gpu(tr, torch, dev, *frame)
+        keep = ~ref["band"]
+        for name in ("down", "up"):
+            assert np.array_equal(g[name][keep], ref[name][keep]), name
     finally:
         tr.close()
