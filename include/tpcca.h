@@ -225,8 +225,9 @@ int tpc_track_timeframe_noalloc(const tpc_tf_config *cfg, const tpc_clusters *cl
 /* tpc_track_timeframe replayed from a CUDA graph (one graph launch per call; the
  * paper has no counterpart).  The first call with a given pair of argument
  * structs captures the call's kernels into a graph owned by the handle; a later
- * call with byte-identical structs (same pointers, n, flags, capacities) and the
- * same tile choice launches that graph; any other call recaptures.  The graph
+ * call with byte-identical structs (same pointers, n, flags, capacities), the same
+ * classifier (tpc_mlp_load) and the same choices of the handle (tpc_tf_autotune,
+ * tpc_tf_set_spin_limit) launches that graph; any other call recaptures.  The graph
  * reads the buffers the structs point to at launch time, so the caller refills
  * them between calls.  out->n_tracks_host must be NULL.  Errors as for
  * tpc_track_timeframe; device-side errors surface through tpc_tf_status. */

@@ -51,6 +51,17 @@ static_assert(kPinnedCounters + kNCounters <= 64, "page-locked words");
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
+// What a captured call holds besides its argument structs: the handle's choices, and the
+// classifier (its standardisation and output layer are kernel parameters).
+struct GraphKey {
+  int nb_tile, fit_variant, mlp_engine;
+  uint32_t spin_limit, mlp_loads;
+  bool operator==(const GraphKey &o) const {
+    return nb_tile == o.nb_tile && fit_variant == o.fit_variant && mlp_engine == o.mlp_engine &&
+           spin_limit == o.spin_limit && mlp_loads == o.mlp_loads;
+  }
+};
+
 }  // namespace
 
 struct tpc_tf {
@@ -109,6 +120,7 @@ struct tpc_tf {
   MlpHead mlp_head = {};      // host copy of the values every scored row reads
   float *mlp_stage = nullptr; // FP32 blob body staged for packing
   bool mlp_ready = false;
+  uint32_t mlp_loads = 0;     // classifiers loaded so far
   float logit_tau = 0.f;
   // track follower (cfg.follow): the chain tracks' fit records, claims, joins and
   // the followed tracks' membership (arena, follow mode only)
@@ -144,7 +156,7 @@ struct tpc_tf {
   cudaGraphExec_t graph_exec = nullptr;
   tpc_clusters graph_cl;
   tpc_tracks graph_out;
-  int graph_nb_tile = 0;
+  GraphKey graph_key = {};
   int graph_launches = 0;
   uint32_t spin_limit = kSpinLimit;  // polls before a look-back wait gives up
 };
@@ -1110,6 +1122,7 @@ extern "C" int tpc_mlp_load(tpc_tf *tf, const void *blob, size_t bytes) {
     tf->mlp_stage = reinterpret_cast<float *>(reinterpret_cast<char *>(tf->mlp) + (mlp_weights_bytes() + 255) / 256 * 256);
     TPC_CK(cudaMemset(tf->mlp, 0, mlp_weights_bytes()));
   }
+  ++tf->mlp_loads;
   TPC_CK(cudaMemcpy(tf->mlp_stage, static_cast<const char *>(blob) + 16, need - 16, cudaMemcpyHostToDevice));
   const float *body = tf->mlp_stage;
   {  // host copy: blob body = mean (12), inv_std (12), theta (W1, b1, W2, b2, w3, b3)
@@ -1207,8 +1220,9 @@ extern "C" int tpc_track_timeframe_graph(tpc_tf *tf, const tpc_clusters *cl, con
   if (out->n_tracks_host)
     return fail(TPC_ERR_ARG, "tpc_track_timeframe_graph: n_tracks_host must be NULL (a graph does not synchronise)");
   TPC_CK(cudaSetDevice(tf->device));
+  const GraphKey key = {tf->nb_tile, tf->cfg.fit_variant, tf->cfg.mlp_engine, tf->spin_limit, tf->mlp_loads};
   const bool same = tf->graph_exec && std::memcmp(&tf->graph_cl, cl, sizeof(*cl)) == 0 &&
-                    std::memcmp(&tf->graph_out, out, sizeof(*out)) == 0 && tf->graph_nb_tile == tf->nb_tile;
+                    std::memcmp(&tf->graph_out, out, sizeof(*out)) == 0 && tf->graph_key == key;
   if (!same) {
     if (tf->graph_exec) {
       cudaGraphExecDestroy(tf->graph_exec);
@@ -1232,7 +1246,7 @@ extern "C" int tpc_track_timeframe_graph(tpc_tf *tf, const tpc_clusters *cl, con
     if (ei != cudaSuccess) return fail(TPC_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(ei));
     tf->graph_cl = *cl;
     tf->graph_out = *out;
-    tf->graph_nb_tile = tf->nb_tile;
+    tf->graph_key = key;
     tf->graph_launches = tf->launches;
   }
   TPC_CK(cudaGraphLaunch(tf->graph_exec, (cudaStream_t)stream));
