@@ -80,7 +80,9 @@ extern "C" {
 
 #define TPC_OK 0
 #define TPC_ERR_ARG (-1)      /* invalid argument (null pointer, bad config, misaligned buffer) */
-#define TPC_ERR_CAPACITY (-2) /* more clusters than max_clusters, or more tracks than track_capacity */
+#define TPC_ERR_CAPACITY (-2) /* more clusters than max_clusters, more tracks than track_capacity, unsorted input
+                                 with more than 16384 clusters in a (sector, row), or a link to a cluster past
+                                 the 65535th of one (the tracks then lack it) */
 #define TPC_ERR_CUDA (-3)     /* a CUDA runtime call failed */
 #define TPC_ERR_INPUT (-4)    /* device validation: sector >= 36, row >= 152, pad or time out of range or
                                  not finite, or input flagged sorted but not sorted */

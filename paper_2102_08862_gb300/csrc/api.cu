@@ -424,6 +424,9 @@ static int map_err(uint32_t w) {
   if (w & kErrTimeout) return fail(TPC_ERR_TIMEOUT, "a bounded device-side wait gave up");
   if (w & kErrSortCap)
     return fail(TPC_ERR_CAPACITY, "unsorted input with more than 16384 clusters in one (sector, row): pass sorted input");
+  // (a long row alone, kErrRowCap, is no error: only a lost link makes the result wrong)
+  if (w & kErrRowLost)
+    return fail(TPC_ERR_CAPACITY, "links to clusters past the 65535th of a (sector, row) were lost");
   if (w & kErrCapacity) return fail(TPC_ERR_CAPACITY, "more tracks than the track capacity");
   if (w & kErrInternal) return fail(TPC_ERR_CUDA, "internal device error");
   return TPC_OK;

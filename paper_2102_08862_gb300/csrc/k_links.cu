@@ -108,7 +108,7 @@ __device__ __forceinline__ void stage_links(const Args &a, uint32_t bid, uint32_
       if (lane == 0 && i < (int)n) a.start_bits[i >> 5] = bits;
     }
   }
-  if (bad) raise(a.ctr, kErrRowCap);
+  if (bad) raise(a.ctr, kErrRowCap | kErrRowLost);
 }
 
 // The set bits of a mask over the clusters in cluster order (the start hits; the

@@ -56,7 +56,8 @@ enum : uint32_t {
   kErrTimeout = 4u,
   kErrInternal = 8u,
   kErrSortCap = 16u,
-  kErrRowCap = 32u  // a (sector, row) with more than 65534 clusters
+  kErrRowCap = 32u,  // a (sector, row) with more than 65534 clusters
+  kErrRowLost = 64u  // a mutual link to a cluster past a row's 65535th, which 16 bits do not hold
 };
 
 // counters at the head of the per-call reset region
