@@ -34,6 +34,7 @@ __device__ __forceinline__ void stage_row_index_table(const Args &a) {
   const int nkeys = a.nkeys, tile = a.nb_tile;
   const int per = (nkeys + 255) / 256, k0 = min(nkeys, tid * per), k1 = min(nkeys, k0 + per);
   const int32_t n = (int32_t)a.n;
+  if (tid == 0) a.key_first[0] = 1u;  // (its keys are read by this thread alone)
   // first present cluster of this thread's keys, then of all keys behind them
   int32_t mine = n;
   for (int k = k0; k < k1; k += kBatch) {
@@ -61,7 +62,7 @@ __device__ __forceinline__ void stage_row_index_table(const Args &a) {
 #pragma unroll
     for (int u = 0; u < kBatch; ++u)
       if (ke - 1 - u >= k0) {
-        const int32_t begin = ke - 1 - u == 0 ? 0 : v[u] ? min(run, (int32_t)v[u] - 1) : run;
+        const int32_t begin = v[u] ? min(run, (int32_t)v[u] - 1) : run;
         const int c = run - begin;
         a.row_begin[ke - 1 - u] = begin;
         mx = max(mx, c);
