@@ -571,7 +571,7 @@ static int enqueue_linking(tpc_tf *tf, const tpc_clusters *cl, Args &a, cudaStre
     stage(tf, st, "sort");
   }
   launch_quantize(a, tf->sms, st);
-  launch_tile_windows(a, st);
+  launch_tile_windows(a, tf->cfg.row_cap, st);
   stage(tf, st, "ingest");
   launch_neighbours(a, tf->cfg.row_cap, tf->sms, st, prune);
   stage(tf, st, "neighbours");

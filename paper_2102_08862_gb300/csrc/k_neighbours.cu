@@ -17,8 +17,8 @@
 // neighbour kernel gives each tile one CTA: the bulk-copy (TMA) engine copies the
 // tile and both windows from the quantised array into shared memory, completion
 // on an mbarrier; then each warp links 32 consecutive clusters at a time, a cluster
-// per lane.  Windows larger than the staging buffers are read from global memory
-// with the same arithmetic.
+// per lane.  A tile whose windows are larger than the staging buffers is cut into parts;
+// windows that are still larger are read from global memory with the same arithmetic.
 //
 // What bounds it: instruction issue (79 % of the slots) and the integer pipe, which
 // takes half of them at half rate; DRAM traffic is 14 of the 16 bytes a cluster
@@ -431,10 +431,62 @@ struct __align__(16) NbSmem {
 }  // namespace
 
 // ------------------------------------------------------------ tile windows
+// A tile with a range of more than win_cap entries (the neighbour kernel's staging
+// buffers) is cut into parts, which become tiles behind the others: halved until every
+// part's ranges fit, down to kNbPart clusters.  The neighbour kernel's grid has as many
+// places as tiles could be needed for any division into rows, and the parts take those
+// that this frame leaves free (one per row is there for a row's last tile, so half of the
+// rows' number on average); a tile that finds none stays whole.  (1 M clusters of one
+// sector at 160 and 200 times the usual density, tile 768, a call: whole tiles, read from
+// global memory, 48.0 and 93.4 ms, parts 6.7 and 8.2; 22.2 and 33.1 with the windows of
+// up to 1279 entries that an earlier form staged.  Parts linked one after the other by
+// the tile's own CTA took 6.7 and 8.7, but the loop cost the usual tiles 1 to 5 %.)
+constexpr int kNbPart = 128;
+// Tile t, clusters [ta, tb) of `key`, whose ranges do not fit: its parts' entries.  Out
+// of line, so that the usual tile's search keeps its registers.
+static __device__ __noinline__ void split_tile(const Args &a, int win_cap, uint32_t t, int key, int ta, int tb) {
+  const int pb = a.row_begin[key - 1], nb = a.row_begin[key + 1], ne = a.row_begin[key + 2], pe = a.row_begin[key];
+  auto windows = [&](int c0, int c1) {
+    const int t0 = a.tq[c0].x - a.wt, t1 = a.tq[c1 - 1].x + a.wt + 1;
+    int4 w;
+    w.x = tq_lower_bound(a.tq, pb, pe, t0);
+    w.y = tq_lower_bound(a.tq, w.x, pe, t1);
+    w.z = tq_lower_bound(a.tq, nb, ne, t0);
+    w.w = tq_lower_bound(a.tq, w.z, ne, t1);
+    return w;
+  };
+  int len = tb - ta;
+  for (bool ok = false; !ok && len > kNbPart;) {
+    len = max(kNbPart, (len + 1) / 2);
+    ok = true;
+    for (int c = ta; ok && c < tb; c += len) {
+      const int4 w = windows(c, min(tb, c + len));
+      ok = w.y - w.x <= win_cap && w.w - w.z <= win_cap;
+    }
+  }
+  const uint32_t places = min(a.n / (uint32_t)a.nb_tile + (uint32_t)a.nkeys + 1u, a.tile_cap);
+  const uint32_t extra = (uint32_t)((tb - ta - 1) / len);
+  uint32_t slot = a.ctr[kCtrTiles], seen;
+  for (;; slot = seen) {
+    if (slot + extra > places) {
+      len = tb - ta;
+      break;
+    }
+    seen = atomicCAS(&a.ctr[kCtrTiles], slot, slot + extra);
+    if (seen == slot) break;
+  }
+  for (int c = ta; c < tb; c += len) {
+    const int end = min(tb, c + len);
+    const uint32_t e = c == ta ? t : slot++;
+    a.tile_win[2 * e] = make_int4(key, c, end, 0);
+    a.tile_win[2 * e + 1] = windows(c, end);
+  }
+}
+
 // One thread per tile: the tile's cluster range and the ranges of rows r-1 and
 // r+1 whose t_q lies in [t_first - wt, t_last + wt].
-__device__ __forceinline__ void stage_tile_windows(const Args &a, uint32_t bid, uint32_t nblk) {
-  const uint32_t ntiles = min(a.ctr[kCtrTiles], a.tile_cap);
+__device__ __forceinline__ void stage_tile_windows(const Args &a, int win_cap, uint32_t bid, uint32_t nblk) {
+  const uint32_t ntiles = min((uint32_t)a.tile_off[a.nkeys], a.tile_cap);
   for (uint32_t t = bid * blockDim.x + threadIdx.x; t < ntiles; t += nblk * blockDim.x) {
     // key = last (sector, row) whose first tile is <= t
     int lo = 0, hi = a.nkeys;
@@ -483,6 +535,10 @@ __device__ __forceinline__ void stage_tile_windows(const Args &a, uint32_t bid, 
         if (!more) break;
       }
       win = make_int4(lo[0], max(lo[1], lo[0]), lo[2], max(lo[3], lo[2]));  // (max: only with unsorted input)
+      if (max(win.y - win.x, win.w - win.z) > win_cap && tb - ta > kNbPart) {
+        split_tile(a, win_cap, t, key, ta, tb);
+        continue;
+      }
     }
     a.tile_win[2 * t] = make_int4(key, ta, max(ta, tb), 0);
     a.tile_win[2 * t + 1] = win;
@@ -661,9 +717,9 @@ __device__ __forceinline__ void stage_edge_claims(const Args &a, uint32_t bid, u
 }
 
 #ifndef TPC_STAGES_ONLY
-__global__ void __launch_bounds__(256) k_tile_windows(Args a) {
+__global__ void __launch_bounds__(256) k_tile_windows(Args a, int win_cap) {
   pdl_begin();
-  stage_tile_windows(a, blockIdx.x, gridDim.x);
+  stage_tile_windows(a, win_cap, blockIdx.x, gridDim.x);
 }
 __global__ void __launch_bounds__(256) k_edge_claims(Args a) {
   pdl_begin();
@@ -671,17 +727,22 @@ __global__ void __launch_bounds__(256) k_edge_claims(Args a) {
 }
 
 // ------------------------------------------------------------------ launchers
-void launch_tile_windows(const Args &a, cudaStream_t st) {
+// entries of a staged window: the variant's capacity, or row_cap if that is smaller
+static int nb_win_cap(const Args &a, int row_cap) {
+  const int cap = (a.nb_tile == 1024 ? 2048 : 1024) - 1;
+  return row_cap > 0 && row_cap < cap ? row_cap : cap;
+}
+
+void launch_tile_windows(const Args &a, int row_cap, cudaStream_t st) {
   const uint32_t tiles = neighbour_tiles_max(a.n, a.nkeys, a.nb_tile);
-  launch_pdl(k_tile_windows, (tiles + 255) / 256, 256, 0, st, a.n, a);
+  launch_pdl(k_tile_windows, (tiles + 255) / 256, 256, 0, st, a.n, a, nb_win_cap(a, row_cap));
 }
 
 template <int TILE, int CAP, int THREADS>
 static void launch_nb(const Args &a, int row_cap, cudaStream_t st, bool prune) {
-  const int cap = row_cap > 0 && row_cap < CAP - 1 ? row_cap : CAP - 1;
   const uint32_t grid = neighbour_tiles_max(a.n, a.nkeys, TILE);
   launch_pdl(prune ? k_neighbours<true, TILE, CAP, THREADS> : k_neighbours<false, TILE, CAP, THREADS>, grid, THREADS, 0, st,
-             a.n, a, cap);
+             a.n, a, nb_win_cap(a, row_cap));
 }
 
 void launch_neighbours(const Args &a, int row_cap, int sms, cudaStream_t st, bool prune) {

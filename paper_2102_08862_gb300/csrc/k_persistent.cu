@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(256, 6) k_track_persistent(Args a, int vec, in
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
   if (bid == 0) stage_row_index_table(a);
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
-  stage_tile_windows(a, bid, nblk);
+  stage_tile_windows(a, win_cap, bid, nblk);
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
   stage_neighbours<false, TILE, CAP, 256>(a, win_cap, bid, nblk);
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;

@@ -181,7 +181,7 @@ extern "C" int tpc_track_timeframe_noalloc(const tpc_tf_config *cfg, const tpc_c
   if (cudaMemsetAsync(a.ctr, 0, reset_bytes, st) != cudaSuccess)
     return report(TPC_ERR_CUDA, "tpc_track_timeframe_noalloc: clearing the counters failed");
   launch_quantize(a, sms, st);
-  launch_tile_windows(a, st);
+  launch_tile_windows(a, 0, st);
   launch_neighbours(a, 0, sms, st);
   launch_edge_claims(a, st);
   launch_links(a, sms, st);

@@ -61,7 +61,7 @@ inline size_t reset_words(int nkeys) { return (size_t)kNCounters + (((size_t)nke
 // validation of every sorted cluster, its quantised (t, y) into a.tq, the (sector, row)
 // index and the tile table
 void launch_quantize(const Args &a, int sms, cudaStream_t st);
-void launch_tile_windows(const Args &a, cudaStream_t st);
+void launch_tile_windows(const Args &a, int row_cap, cudaStream_t st);
 // prune = true also lists the clusters with >= 2 pairs under the cost cut in a.amb
 // row_cap > 0 lowers the staged window capacity (tests of the global-memory path)
 void launch_neighbours(const Args &a, int row_cap, int sms, cudaStream_t st, bool prune = false);
