@@ -515,9 +515,13 @@ void launch_fit(const Args &a, int sms, int variant, cudaStream_t st) {
 
 void launch_fit_assign(const Args &a, int sms, cudaStream_t st) {
   // a block per 256-track group, as above, up to one track in 48 clusters (they average
-  // 70); denser frames take groups in turn.  Empty blocks would only delay the assignment.
+  // 70) and up to one block per SM whatever the chains' length; denser frames take groups
+  // in turn.  More empty blocks would only delay the assignment.  (Chains of 3 to 5
+  // clusters, n_min 3, us a call, without the blocks per SM -> with them: 60 k clusters
+  // 127 -> 97, 300 k 150 -> 121; 2 or 4 per SM the same.)
   const size_t groups = ((size_t)a.track_list_cap + kFitThreads - 1) / kFitThreads;
-  const size_t usual = (size_t)a.n / (48 * kFitThreads) + 1;
+  const size_t by_size = (size_t)a.n / (48 * kFitThreads) + 1;
+  const size_t usual = by_size > (size_t)sms ? by_size : (size_t)sms;
   const uint32_t fit = (uint32_t)(groups < usual ? (groups ? groups : 1) : usual);
   k_fit_assign<<<fit + assign_blocks(a, sms), kFitThreads, kFitAssignCap * 4, st>>>(a, fit);
 }
