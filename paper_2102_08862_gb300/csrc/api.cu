@@ -398,6 +398,13 @@ extern "C" int tpc_tf_create(const tpc_tf_config *cfg, tpc_tf **out) {
     off += align_up(p.bytes, 256);
   }
   tf->sort_scratch_bytes = sort_scratch_bytes(tf->N);
+  // the hit removal's counter starts at zero (its kernel leaves it so), and the status is good
+  e = cudaMemsetAsync(tf->reset, 0, kNCounters * 4, tf->side_stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(tf->side_stream);
+  if (e != cudaSuccess) {
+    free_all(tf);
+    return fail(TPC_ERR_CUDA, std::string("clearing the counters: ") + cudaGetErrorString(e));
+  }
   e = cudaMallocHost(&tf->pinned, 256);
   if (e != cudaSuccess) {
     free_all(tf);
@@ -1361,8 +1368,6 @@ extern "C" int tpc_tf_remove_unassigned(tpc_tf *tf, const tpc_clusters *cl, cons
   cudaStream_t st = (cudaStream_t)stream;
   Args a;
   fill_args(tf, n, nullptr, a);
-  // the compaction's counter (the error word stays)
-  TPC_CK(cudaMemsetAsync(tf->reset + kCtrCompactTile, 0, 4, st));
   launch_compact(a, cl->sector, cl->row, cl->pad, cl->time, cluster_track, sector, row, pad, time, track, count,
                  tf->sms, st);
   TPC_CK(cudaGetLastError());

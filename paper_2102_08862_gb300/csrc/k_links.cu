@@ -343,6 +343,9 @@ __global__ void __launch_bounds__(kThreads) k_assign(Args a) {
 // the counts into offsets; k_compact then copies each tile on its own: a warp holds 256
 // consecutive clusters, 32 at a time, so that loads are coalesced and the kept ones of a
 // round go to consecutive places.  No tile waits for another.
+// The counter of the finished CTAs is zero between calls: the last CTA puts it back, so
+// that a small call needs no memset (24 us with one and a full launch gap before the
+// copies, 7600 clusters, host and device; 22.9 so; 22.4 in one pass).
 // What bounds it: memory, 4 + 16 B per cluster and 16 per kept one.  16.8 M clusters,
 // 90 % kept: 0.125 ms (k_compact 0.086, 5.8 TB/s).  An ordered compaction in one pass
 // (each tile's fields loaded once a look-back had told its place, staged in shared
@@ -350,6 +353,7 @@ __global__ void __launch_bounds__(kThreads) k_assign(Args a) {
 __global__ void __launch_bounds__(kThreads) k_compact_count(uint32_t n, const int32_t *__restrict__ ct, int vec,
                                                             uint32_t *__restrict__ offset, uint32_t *o_count,
                                                             uint32_t *ctr) {
+  pdl_begin();
   __shared__ uint32_t s_warp[kThreads / 32];
   __shared__ bool s_last;
   const uint32_t n_tiles = (n + kLinkTile - 1) / kLinkTile;
@@ -400,7 +404,10 @@ __global__ void __launch_bounds__(kThreads) k_compact_count(uint32_t n, const in
       run += v[u];
     }
   }
-  if (threadIdx.x == 0) *o_count = total;
+  if (threadIdx.x == 0) {
+    *o_count = total;
+    ctr[kCtrCompactTile] = 0;  // (all CTAs have counted: the next call finds it as this one did)
+  }
 }
 
 __global__ void __launch_bounds__(kThreads) k_compact(uint32_t n, const uint16_t *__restrict__ sector,
@@ -410,6 +417,7 @@ __global__ void __launch_bounds__(kThreads) k_compact(uint32_t n, const uint16_t
                                                       uint16_t *__restrict__ o_sector, uint16_t *__restrict__ o_row,
                                                       float *__restrict__ o_pad, float *__restrict__ o_time,
                                                       int32_t *__restrict__ o_track) {
+  pdl_begin();
   constexpr int kWarps = kThreads / 32, kRounds = kLinkTile / kThreads;
   __shared__ uint32_t s_cnt[kWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -465,8 +473,8 @@ void launch_compact(const Args &a, const uint16_t *sector, const uint16_t *row, 
   k_compact_count<<<blocks < cap ? (blocks ? blocks : 1u) : cap, kThreads, 0, st>>>(
       a.n, ct, ((uintptr_t)ct & 15) == 0 ? 1 : 0, offset, o_count, a.ctr);
   if (tiles > 0)
-    k_compact<<<tiles, kThreads, 0, st>>>(a.n, sector, row, pad, time, ct, offset, o_sector, o_row, o_pad, o_time,
-                                          o_track);
+    launch_pdl(k_compact, tiles, kThreads, 0, st, a.n, a.n, sector, row, pad, time, ct, offset, o_sector, o_row, o_pad,
+               o_time, o_track);
 }
 
 // inspection: the mutual up link as a sorted position, and the start flag

@@ -103,8 +103,8 @@ int launch_sort(const Args &a, const uint16_t *sector, const uint16_t *row, cons
                 uint16_t *s_sector, uint16_t *s_row, float *s_pad, float *s_time, int32_t *perm, void *scratch,
                 size_t scratch_bytes, void *records, size_t records_bytes, int sms, cudaStream_t st);
 size_t sort_scratch_bytes(uint32_t max_n);
-// hit removal: clusters with ct >= 0 in caller order (uses a.lb_links and a.ctr,
-// which must be cleared)
+// hit removal: clusters with ct >= 0 in caller order (a.lb_links holds its tiles'
+// offsets; its counter in a.ctr must be zero and is zero again afterwards)
 void launch_compact(const Args &a, const uint16_t *sector, const uint16_t *row, const float *pad, const float *time,
                     const int32_t *ct, uint16_t *o_sector, uint16_t *o_row, float *o_pad, float *o_time,
                     int32_t *o_track, uint32_t *o_count, int sms, cudaStream_t st);
