@@ -191,8 +191,7 @@ __global__ void __launch_bounds__(kPruneWarps * 32) k_prune(Args a, const MlpW *
   };
   for (uint32_t e = blockIdx.x * kPruneWarps + warp; e < n_amb; e += gridDim.x * kPruneWarps) {
     const int4 en = a.amb[e];
-    const int i = en.x, jlo = en.y, klo = en.z;
-    const int row_key = key_at<false>(a, a.row_begin, i), r = row_key % kNRows;
+    const int i = en.x, jlo = en.y, klo = en.z, row_key = en.w, r = row_key % kNRows;
     const int2 ci = ty_of(a, i, r);
     const int ti = ci.x, yi = ci.y;
     const int jend = a.row_begin[row_key], kend = a.row_begin[row_key + 2];  // (listed clusters: 1 <= r <= 150)

@@ -65,8 +65,11 @@ __device__ __forceinline__ int tq_lower_bound(const int2 *tq, int lo, int hi, in
 
 
 // Pruned mode: append a cluster with >= 2 pairs under the cost cut to the list
-// the classifier rescores.  The lanes that append together share one atomic.
-__device__ __forceinline__ void amb_push(const Args &a, int4 e) {
+// the classifier rescores: its position, the first entries of its windows and its
+// (sector, row), which is its tile's (pruned mode has a CTA per tile).  The lanes that
+// append together share one atomic.
+__device__ __forceinline__ void amb_push(const Args &a, int i, int j0, int k0) {
+  const int4 e = make_int4(i, j0, k0, a.tile_win[2 * blockIdx.x].x);
   const unsigned m = __activemask();
   const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
   uint32_t base = 0;
@@ -196,7 +199,7 @@ __device__ __noinline__ void link_run(const Args &a, int li0, int li1, int cnt, 
       }
     }
     out[li] = (bj >= 0 && best <= cost_max) ? make_int2(base_p + bj, base_n + bk) : make_int2(-1, -1);
-    if (kPrune && nc >= 2) amb_push(a, make_int4(base_c + li, base_p + jlo, base_n + klo, nc));
+    if (kPrune && nc >= 2) amb_push(a, base_c + li, base_p + jlo, base_n + klo);
   }
 }
 
@@ -379,7 +382,7 @@ __device__ __forceinline__ void link_tile_smem(const Args &a, int cnt, const int
         }
       } else {
         if (nc <= kPruneMaxPairs && row <= kPruneRegionRows) q->end = old;  // the first that does not fit
-        amb_push(a, make_int4(base_c + li, j0, k0, nc));
+        amb_push(a, base_c + li, j0, k0);
       }
     }
   }

@@ -144,7 +144,7 @@ struct Args {
   uint32_t *n_tracks_out;
   // pruned mode: clusters whose pairs the link classifier rescores outside the
   // neighbour kernel (windows not staged, or the kernel's queue full)
-  int4 *amb;               // (sorted position, first j of the window, first k of the window, pairs under the cut)
+  int4 *amb;               // (sorted position, first j of the window, first k of the window, (sector, row))
   uint32_t amb_cap;
   const struct MlpW *mlp;  // packed classifier weights
   float logit_tau;         // a pair is kept when its logit >= logit_tau
