@@ -41,12 +41,12 @@ STAGED_BYTES_PER_CLUSTER = 48.0
 IO_FLOOR_BYTES_PER_CLUSTER = 16.0  # 12 B of cluster fields in, 4 B of cluster_track out
 NOMINAL_HBM_GBS = 8000.0
 FIT_FLOP_PER_CLUSTER = 200.0  # transport + 2-D update per cluster in a track (algorithmic)
-# DRAM bytes per cluster of k_neighbours from one full ncu capture of the 5 ms frame,
+# DRAM bytes per cluster of k_neighbours from ncu captures of the 5 ms frame,
 # valid while k_neighbours.cu is the file captured (its SHA-256)
-NB_TRAFFIC = {"sha256": "6e1379e7dbaee8819b9d3525c7d5f9fb4f5df8618ad9713a9f60a67441c45300",
-              "pruned": (134974208 + 102912256) / 16765809, "plain": (134964224 + 94144768) / 16765809}
+NB_TRAFFIC = {"sha256": "d66143d4270c6ceff6606e97b904d380f8c63f27b3bf0639557aa0772cccf5a5",
+              "pruned": (134959616 + 102696960) / 16765809, "plain": (134947840 + 94069504) / 16765809}
 # warp instructions per cluster of the same captures (smsp__inst_executed.sum / clusters)
-NB_INST = {"pruned": 259034661 / 16765809, "plain": 221510458 / 16765809}
+NB_INST = {"pruned": 259029897 / 16765809, "plain": 221514637 / 16765809}
 
 
 def neighbours_traffic(mode, n):

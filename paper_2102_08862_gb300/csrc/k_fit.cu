@@ -406,7 +406,8 @@ __global__ void __launch_bounds__(kFitThreads) k_fit_thread(Args a) { stage_fit<
 // 2 ms frame to 0.57 ms.)
 // clusters of a row built in shared memory at once: 26 KB holds a row of a 10 ms frame
 // and leaves the fit its L1 cache (10 ms frame, a call: 16 KB 1632 us, 26 KB 1559, 32 KB
-// 1574, 48 KB 2149)
+// 1574, 48 KB 2149).  Longer rows take two or more chunks: frames of 12, 16, 20 and 25 ms
+// take 1652, 2157, 2617 and 3397 us, in proportion to their clusters.
 constexpr int kFitAssignCap = 6656;
 __global__ void __launch_bounds__(kFitThreads) k_fit_assign(Args a, uint32_t fit_blocks) {
   extern __shared__ int32_t assign_buf[];

@@ -42,8 +42,8 @@ constexpr uint16_t kNone16 = 0xffff;
 // partners' links (the partners of neighbours in time are neighbours too), touch a few
 // lines each.  Steps share nothing and need no barrier, so that the dependent loads
 // (link, partners' links) of 64 warps overlap.
-// What bounds it: the latency of those two loads and the instructions between them (58
-// % of the issue slots); 2.6 TB/s of DRAM traffic.  An earlier form gave a thread 8
+// What bounds it: the latency of those two loads and the instructions between them (63
+// % of the issue slots); 2.7 TB/s of DRAM traffic.  An earlier form gave a thread 8
 // consecutive clusters (every lane of a gather met a line of its own) and compacted the
 // start hits in the same pass: 0.27 ms on the 10 ms frame, 0.061 on 2 ms.  With
 // coalesced gathers alone it took 0.25: the barriers around each tile's look-back were

@@ -461,12 +461,14 @@ __device__ __forceinline__ void tc_put_input_c(unsigned char *x, int r, const fl
 // threads holds two 128-row tiles, warpgroup h (threads 128 h ..) tile h, thread r of it
 // row r (tensor-memory lane r, columns 64 h ..).  The warpgroups share the staged
 // weights only: each issues its own MMAs, waits on its own mbarrier and meets at its own
-// named barrier, so that one's epilogue runs while the other's MMAs do (5.2 M rows: both
-// tiles in step 111.1 us, so 109.9; with the output layer's multiply-adds one by one
-// instead of in pairs 113.4).  The next step's row is loaded while the current step runs.  4 CTAs share an SM (tensor memory: 4 x 128 of
-// 512 columns; 64 registers a thread), 32 warps in all, which hide the MMA and load
-// latencies; the per-row constants are kernel parameters (MlpHead), so the epilogues
-// read no shared memory.
+// named barrier, so that one's epilogue runs while the other's MMAs do.  5.2 M rows: 108.3
+// us, 113.5 with both tiles in step and the output layer's multiply-adds one by one (timed
+// in turn; on another GB300 109.9, against 111.1 in step and 113.4 with single multiply-adds).
+// What bounds it: a tile's serial chain, inputs, MMA, epilogue, MMA, epilogue; issue slots
+// 59 % active, the ALU pipe 54 %, tensor 26 %.  The next step's row is loaded while the
+// current step runs.  4 CTAs share an SM (tensor memory: 4 x 128 of 512 columns; 64
+// registers a thread), 32 warps in all, which hide part of the MMA and load latencies; the
+// per-row constants are kernel parameters (MlpHead), so the epilogues read no shared memory.
 // With m_dev set, the rows are the first min(*m_dev, m) (a count written on the
 // device by an earlier kernel of the stream; m is then the buffers' capacity).
 __global__ void __launch_bounds__(256, 4) k_mlp_score_tc(const MlpW *__restrict__ W, const __grid_constant__ MlpHead hd,

@@ -439,11 +439,11 @@ struct __align__(16) NbSmem {
 // part's ranges fit, down to kNbPart clusters.  The neighbour kernel's grid has as many
 // places as tiles could be needed for any division into rows, and the parts take those
 // that this frame leaves free (one per row is there for a row's last tile, so half of the
-// rows' number on average); a tile that finds none stays whole.  (1 M clusters of one
+// rows' number on average); a tile that finds none stays whole.  1 M clusters of one
 // sector at 160 and 200 times the usual density, tile 768, a call: whole tiles, read from
-// global memory, 48.0 and 93.4 ms, parts 6.7 and 8.2; 22.2 and 33.1 with the windows of
-// up to 1279 entries that an earlier form staged.  Parts linked one after the other by
-// the tile's own CTA took 6.7 and 8.7, but the loop cost the usual tiles 1 to 5 %.)
+// global memory, 48 and 90 ms; parts 6.7 and 8.3; windows of up to 1279 entries, which an
+// earlier form staged, 22 and 33.  Parts linked one after the other by the tile's own CTA
+// took 6.7 and 8.7, but the loop cost the usual tiles 1 to 5 %.
 constexpr int kNbPart = 128;
 // Tile t, clusters [ta, tb) of `key`, whose ranges do not fit: its parts' entries.  Out
 // of line, so that the usual tile's search keeps its registers.
