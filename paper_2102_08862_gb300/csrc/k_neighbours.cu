@@ -599,13 +599,14 @@ __device__ __forceinline__ void nb_tile(const Args &a, int win_cap, uint32_t t, 
     if (bn) bulk_g2s(sm.n, a.tq + n0, bn, &sm.bar);
   }
   // bounded wait for the copies; if any thread gives up, the CTA records a
-  // timeout, waits once more (bounded) for copies still in flight and leaves the
-  // tile unlinked (the decision is taken by the whole CTA at one barrier)
+  // timeout, waits once more (bounded) for copies still in flight and gives the tile
+  // no links (the decision is taken by the whole CTA at one barrier).  The limit is
+  // not the handle's: a CTA must not end with copies into its shared memory in flight.
   bool ok = true;
   const uint32_t ph = phase;
   phase ^= 1u;
   for (uint32_t it = 0; !mbar_try(&sm.bar, ph); ++it) {  // try_wait suspends the thread for a while itself
-    if (it >= a.spin_limit) {
+    if (it >= kSpinLimit) {
       ok = false;
       break;
     }
@@ -620,8 +621,10 @@ __device__ __forceinline__ void nb_tile(const Args &a, int win_cap, uint32_t t, 
   if (__syncthreads_or(!ok)) {
     if (tid == 0) raise(a.ctr, kErrTimeout);
     if (!ok)
-      for (uint32_t it = 0; it < a.spin_limit && !mbar_try(&sm.bar, ph); ++it) {
+      for (uint32_t it = 0; it < kSpinLimit && !mbar_try(&sm.bar, ph); ++it) {
       }
+    if (kPrune && tid == 0) a.q_count[t] = 0;
+    for (int e = tid; e < cnt; e += NT) a.link[ta + e] = make_int2(-1, -1);
     return;
   }
   if (staged) {
