@@ -118,8 +118,9 @@ typedef struct {
   int32_t device;        /* CUDA device ordinal */
   int32_t fit_variant;   /* TPC_FIT_THREAD or TPC_FIT_WARP */
   int32_t profile_stages;/* nonzero: record CUDA events between stages (tpc_tf_stage_times) */
-  int32_t row_cap;       /* clusters per staged row in the neighbour kernel (0: largest that fits
-                            shared memory); rows above it take the global-memory kernel */
+  int32_t row_cap;       /* entries of a staged time window in the neighbour kernel (0: largest that fits
+                            shared memory); tiles with larger windows are cut into parts, and windows
+                            still larger are read from global memory */
   int32_t n_sectors;     /* independent sectors per call (0: the TPC's 36).  A batched call packs
                             many instances (one sector of one time frame each) into one call: the
                             `sector` field of a cluster is then its instance id, < n_sectors <= 16384,
@@ -298,9 +299,10 @@ int tpc_tf_launches_per_call(const tpc_tf *tf);
  * TPC_ERR_ARG (null or misaligned pointer), TPC_ERR_CUDA. */
 int tpc_debug_quantize(const float *v, uint32_t n, int32_t *q, void *stream);
 
-/* Polls after which a device-side look-back wait of this handle gives up and
- * records TPC_ERR_TIMEOUT (the kernel then finishes with a zero prefix, so the
- * context stays usable).  0 restores the default (4194304 polls with a short
+/* Polls after which a device-side look-back or grid-barrier wait of this handle
+ * gives up and records TPC_ERR_TIMEOUT (the call then ends without following the
+ * lists that the wait left incomplete: its results are not valid, the context and
+ * the handle stay usable).  0 restores the default (4194304 polls with a short
  * sleep each).  For tests of the failure path; lower limits can make regular calls
  * report TPC_ERR_TIMEOUT under load.  Errors: TPC_ERR_ARG. */
 int tpc_tf_set_spin_limit(tpc_tf *tf, uint32_t polls);

@@ -27,7 +27,7 @@ constexpr int kAssignBatch = 3;  // groups of 8 tracks a thread loads per round
 template <int kCap>
 __device__ __forceinline__ void stage_assign(const Args &a, uint32_t bid, uint32_t nblk, int32_t *buf) {
   const size_t stride = a.track_list_cap;
-  const uint32_t nl = min(a.ctr[kCtrTracks], a.track_list_cap);
+  const uint32_t nl = listed(a, kCtrTracks, a.track_list_cap);
   for (uint32_t key = bid; key < (uint32_t)a.nkeys; key += nblk) {
     const int rb = a.row_begin[key], re = a.row_begin[key + 1];
     const uint32_t sec = key / kNRows;

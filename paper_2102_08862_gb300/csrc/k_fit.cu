@@ -293,10 +293,13 @@ __device__ __forceinline__ void kf_covariance(const Kf &k, float *c) {
 // shared memory (bitonic), so that the lanes of a warp fit chains of similar
 // length and finish together; the chain reads of a step stay inside the block's
 // 256 columns (1 KB, cached in L1).
-template <int THREADS>
+// kGate: no track after a wait that gave up (the kernels of their own, in which no other
+// wait runs; the persistent kernel has looked before).
+template <int THREADS, bool kGate>
 __device__ __forceinline__ void stage_fit(const Args &a, uint32_t bid, uint32_t nblk) {
   __shared__ uint32_t s_key[THREADS];
-  const uint32_t nt = min(min(a.ctr[kCtrTracks], a.track_list_cap), a.track_capacity);
+  const uint32_t nl = kGate ? listed(a, kCtrTracks, a.track_list_cap) : min(a.ctr[kCtrTracks], a.track_list_cap);
+  const uint32_t nt = min(nl, a.track_capacity);
   const size_t stride = a.track_list_cap;
   for (uint32_t t0 = bid * THREADS; t0 < nt; t0 += nblk * THREADS) {
     {
@@ -393,7 +396,9 @@ __device__ __forceinline__ void stage_fit(const Args &a, uint32_t bid, uint32_t 
 // coalesced chain loads do not pay back: the thread kernel stays the default.
 #ifndef TPC_STAGES_ONLY
 constexpr int kFitThreads = 256;
-__global__ void __launch_bounds__(kFitThreads) k_fit_thread(Args a) { stage_fit<kFitThreads>(a, blockIdx.x, gridDim.x); }
+__global__ void __launch_bounds__(kFitThreads) k_fit_thread(Args a) {
+  stage_fit<kFitThreads, true>(a, blockIdx.x, gridDim.x);
+}
 
 // The fit, then the cluster_track assignment, which reads the same chains: one launch
 // whose first fit_blocks blocks fit and whose others assign.  The fit is the longer
@@ -411,13 +416,13 @@ __global__ void __launch_bounds__(kFitThreads) k_fit_thread(Args a) { stage_fit<
 constexpr int kFitAssignCap = 6656;
 __global__ void __launch_bounds__(kFitThreads) k_fit_assign(Args a, uint32_t fit_blocks) {
   extern __shared__ int32_t assign_buf[];
-  if (blockIdx.x < fit_blocks) stage_fit<kFitThreads>(a, blockIdx.x, fit_blocks);
+  if (blockIdx.x < fit_blocks) stage_fit<kFitThreads, true>(a, blockIdx.x, fit_blocks);
   else stage_assign<kFitAssignCap>(a, blockIdx.x - fit_blocks, gridDim.x - fit_blocks, assign_buf);
 }
 
 __global__ void __launch_bounds__(256) k_fit_warp(Args a) {
   pdl_begin();
-  const uint32_t nt = min(min(a.ctr[kCtrTracks], a.track_list_cap), a.track_capacity);
+  const uint32_t nt = min(listed(a, kCtrTracks, a.track_list_cap), a.track_capacity);
   const size_t stride = a.track_list_cap;
   const int lane = threadIdx.x & 31;
   const uint32_t warps = gridDim.x * (blockDim.x >> 5);
@@ -660,6 +665,11 @@ __global__ void __launch_bounds__(kFollowTileN) k_follow_fit(Args a) {
   __shared__ uint32_t s_key[kFollowTileN], s_excl[kFollowTileN];
   const uint32_t nt = min(a.ctr[kCtrTracks], a.track_list_cap);
   const uint32_t n_tiles = (nt + kFollowTileN - 1) / kFollowTileN;
+  __shared__ bool s_gone;  // a wait before this kernel gave up: no tracks (thread 0's)
+  if (threadIdx.x == 0) {
+    s_gone = timed_out(a);
+    if (s_gone && blockIdx.x == 0 && a.n_tracks_out) *a.n_tracks_out = 0;
+  }
   if (n_tiles == 0) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       a.ctr[kCtrFollowTracks] = 0;
@@ -668,7 +678,7 @@ __global__ void __launch_bounds__(kFollowTileN) k_follow_fit(Args a) {
     return;
   }
   for (;;) {
-    if (threadIdx.x == 0) s_tile = atomicAdd(&a.ctr[kCtrFollowPathTile], 1u);
+    if (threadIdx.x == 0) s_tile = s_gone ? ~0u : atomicAdd(&a.ctr[kCtrFollowPathTile], 1u);
     __syncthreads();
     const uint32_t tile = s_tile;
     if (tile >= n_tiles) break;

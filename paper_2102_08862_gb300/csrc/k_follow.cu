@@ -239,7 +239,7 @@ __device__ __forceinline__ void fs_load(const Args &a, uint32_t t, Fs &f) {
 // the lanes of a warp stay busy together although their follows differ in length.
 __global__ void __launch_bounds__(kThreads) k_follow(Args a) {
   __shared__ int32_t s_rb[kNKeys + 1];
-  const uint32_t nt = min(a.ctr[kCtrTracks], a.track_list_cap);
+  const uint32_t nt = listed(a, kCtrTracks, a.track_list_cap);
   const size_t stride = a.track_list_cap;
   const bool smem_rb = a.nkeys <= kNKeys;
   if (smem_rb)
@@ -664,7 +664,7 @@ __global__ void __launch_bounds__(kSearchThreads) k_sector_search(Args a) {
   // the row after next needs and touches the next row's first probe, so that its
   // search finds both there (a long search's passes follow one another: their
   // latency is the kernel's)
-  const int nf = (int)min(a.ctr[kCtrFirsts], a.starts_cap);
+  const int nf = (int)listed(a, kCtrFirsts, a.starts_cap);
   const int32_t *bound = a.fl.row_first;
   int b0 = 0, b1 = 0, b2 = 0, key = 0;
   auto row_bound = [&](int k) { return min(max(bound[min(k, a.nkeys)], 0), nf); };
@@ -754,7 +754,7 @@ __global__ void __launch_bounds__(kThreads) k_sector_links_resolve(Args a) {
 // Times and tracks of the listed first clusters, and each (sector, row)'s part of the
 // list: an entry fills row_first from behind its predecessor's key up to its own.
 __global__ void __launch_bounds__(kThreads) k_first_index(Args a) {
-  const int nf = (int)min(a.ctr[kCtrFirsts], a.starts_cap), nkeys = a.nkeys;
+  const int nf = (int)listed(a, kCtrFirsts, a.starts_cap), nkeys = a.nkeys;
   auto key_of = [&](int e) {
     const int32_t c = a.starts[e];
     return min((int)a.sector[c] * kNRows + (int)a.row[c], nkeys - 1);

@@ -171,6 +171,11 @@ __device__ __forceinline__ void stage_walk(const Args &a, uint32_t bid) {
   __shared__ uint32_t s_tile, s_prefix;
   __shared__ uint32_t s_warp[kThreads / 32];
   const uint32_t ns = min(a.ctr[kCtrStarts], a.starts_cap);
+  __shared__ bool s_gone;  // the start list's wait gave up: no chains (thread 0's; in shared memory for its register)
+  if (threadIdx.x == 0) {
+    s_gone = timed_out(a);
+    if (s_gone && bid == 0 && a.n_tracks_out) *a.n_tracks_out = 0;
+  }
   const uint32_t n_tiles = (ns + kWalkTileN - 1) / kWalkTileN;
   if (n_tiles == 0) {
     if (bid == 0 && threadIdx.x == 0) {
@@ -199,7 +204,7 @@ __device__ __forceinline__ void stage_walk(const Args &a, uint32_t bid) {
   };
   constexpr int C = kWalkChains;
   for (;;) {
-    if (threadIdx.x == 0) s_tile = atomicAdd(&a.ctr[kCtrTileKeep], 1u);
+    if (threadIdx.x == 0) s_tile = s_gone ? ~0u : atomicAdd(&a.ctr[kCtrTileKeep], 1u);
     __syncthreads();
     const uint32_t tile = s_tile;
     if (tile >= n_tiles) break;

@@ -92,8 +92,12 @@ __global__ void __launch_bounds__(256, 6) k_track_persistent(Args a, int vec, in
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
   stage_walk<false>(a, bid);
   if (!grid_sync(a.ctr, nblk, a.spin_limit)) return;
+  __shared__ bool s_gone;  // the walk's wait gave up (looked at behind the assignment)
+  if (threadIdx.x == 0) s_gone = timed_out(a);
   stage_assign<0>(a, bid, nblk, nullptr);  // (reads the chains, as the fit does: no barrier between them)
-  stage_fit<256>(a, bid, nblk);
+  __syncthreads();
+  if (s_gone) return;
+  stage_fit<256, false>(a, bid, nblk);
 }
 
 int g_pers_blocks[64][3];  // [device][tile variant]: resident CTAs per SM (0: not yet known)

@@ -185,6 +185,17 @@ struct __align__(16) PruneRec {
   uint32_t mj, mk, cn, pad;
 };
 
+// A wait of this call has given up: the ordered compaction it belongs to went on with a
+// prefix that was too small, so entries of its list may be unwritten, and those that read
+// the list take none.  Threads of a CTA may see it differ while another CTA's wait gives up,
+// so that what a CTA decides by it together comes from one thread.
+__device__ __forceinline__ bool timed_out(const Args &a) { return (a.ctr[kCtrErr] & kErrTimeout) != 0; }
+// entries of a list to read (both words are loaded before either is looked at)
+__device__ __forceinline__ uint32_t listed(const Args &a, int counter, uint32_t cap) {
+  const uint32_t err = a.ctr[kCtrErr], count = a.ctr[counter];
+  return err & kErrTimeout ? 0u : min(count, cap);
+}
+
 __device__ __forceinline__ int32_t caller_index(const Args &a, int32_t i) { return a.perm ? a.perm[i] : i; }
 
 // ------------------------------------------------- row of a position
