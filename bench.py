@@ -43,10 +43,10 @@ NOMINAL_HBM_GBS = 8000.0
 FIT_FLOP_PER_CLUSTER = 200.0  # transport + 2-D update per cluster in a track (algorithmic)
 # DRAM bytes per cluster of k_neighbours from ncu captures of the 5 ms frame,
 # valid while k_neighbours.cu is the file captured (its SHA-256)
-NB_TRAFFIC = {"sha256": "d66143d4270c6ceff6606e97b904d380f8c63f27b3bf0639557aa0772cccf5a5",
-              "pruned": (134959616 + 102696960) / 16765809, "plain": (134947840 + 94069504) / 16765809}
+NB_TRAFFIC = {"sha256": "881084a837641b964f91d84da5d8b069912604699c5291e83195e42b6779598a",
+              "pruned": (135078400 + 102718976) / 16765809, "plain": (134950144 + 93987328) / 16765809}
 # warp instructions per cluster of the same captures (smsp__inst_executed.sum / clusters)
-NB_INST = {"pruned": 259029897 / 16765809, "plain": 221514637 / 16765809}
+NB_INST = {"pruned": 258941925 / 16765809, "plain": 221418720 / 16765809}
 
 
 def neighbours_traffic(mode, n):
